@@ -162,8 +162,9 @@ dcp_status dcp_add_map(dcp_graph g, int32_t op, int32_t n_in, const dcp_value* i
  * o_k = offsets[k*ndim .. k*ndim+ndim-1] (axis order as the shape, last
  * axis contiguous), boundary rule `bc`.  Floating dtypes, 1..3 axes,
  * 1 <= npoints <= 32, |offset| <= 4 per axis, steps >= 0.  Rounding: each
- * step is one multiply and FMAs in point order, except on a deferred common
- * weight: a run of two or more steps with a zero or periodic boundary whose
+ * step is one multiply and FMAs, in point order (3 axes) or row by row of the
+ * neighbourhood (1 and 2 axes: ascending offset along the first axis, point
+ * order within a row), except on a deferred common weight: a run of two or more steps with a zero or periodic boundary whose
  * weights are exact multiples of one weight f sums the exact ratios w_k / f
  * and applies f^m every m steps, m bounded so that the scaled state grows by
  * at most 2^32 (float64 only).  Such a run keeps finite results for inputs

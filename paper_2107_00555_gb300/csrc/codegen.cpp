@@ -3,6 +3,7 @@
 // specialised with the group's expression DAG, stencil weights, tile shape
 // and boundary rule.  The expression is emitted as straight-line code in
 // registers; constants are emitted bit-exactly.
+#include <algorithm>
 #include <cfloat>
 #include <cinttypes>
 #include <cstdint>
@@ -11,6 +12,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <sstream>
 
 #include "dcp_internal.h"
@@ -118,6 +120,84 @@ std::string map_expr(const GraphImpl& g, int v, const std::string& a, const std:
   return op_expr(n.op, n.dtype, n.imm, a, b);
 }
 
+// Maps inside stencil kernels (prologues, step epilogues, the tiled reverse's
+// derivatives) are emitted with explicit rounding: a product that feeds an add
+// or a subtraction becomes one fused multiply-add, everything else rounds on
+// its own.  Left to the compiler, that choice depends on how a kernel's blocks
+// are cut, and the kernel forms of one program would differ in last bits.
+struct Ex {
+  std::string s;      // the value
+  std::string x, y;   // a product: s = (neg ? -1 : 1) x y
+  bool neg = false;
+  int uses = 1;
+  bool mul() const { return !x.empty(); }
+};
+
+Ex ex_op(int op, int dtype, double imm_v, const Ex& a, const Ex& b) {
+  const std::string imm = imm_literal(dtype, imm_v);
+  Ex r;
+  auto product = [&](const std::string& x, const std::string& y) {
+    r.s = "dcp_mul_rn(" + x + ", " + y + ")";
+    r.x = x;
+    r.y = y;
+  };
+  // p + q or p - q
+  auto sum = [&](const Ex& p, const Ex& q, bool minus) {
+    auto neg = [](const std::string& v, bool n) { return n ? "dcp_neg(" + v + ")" : v; };
+    if (p.mul() && !(q.mul() && q.uses < p.uses))
+      r.s = "dcp_fma_rn(" + neg(p.x, p.neg) + ", " + p.y + ", " + neg(q.s, minus) + ")";
+    else if (q.mul())
+      r.s = "dcp_fma_rn(" + neg(q.x, q.neg != minus) + ", " + q.y + ", " + p.s + ")";
+    else
+      r.s = std::string(minus ? "dcp_sub_rn(" : "dcp_add_rn(") + p.s + ", " + q.s + ")";
+  };
+  Ex c;
+  c.s = imm;
+  switch (op) {
+    case DCP_MUL: product(a.s, b.s); break;
+    case DCP_MUL_S: product(a.s, imm); break;
+    case DCP_SQUARE: product(a.s, a.s); break;
+    case DCP_NEG:
+      r.s = "dcp_neg(" + a.s + ")";
+      r.x = a.x;
+      r.y = a.y;
+      r.neg = !a.neg;
+      break;
+    case DCP_ADD: sum(a, b, false); break;
+    case DCP_SUB: sum(a, b, true); break;
+    case DCP_ADD_S: sum(a, c, false); break;
+    case DCP_SUB_S: sum(a, c, true); break;
+    case DCP_RSUB_S: sum(c, a, true); break;
+    default: r.s = op_expr(op, dtype, imm_v, a.s, b.s);
+  }
+  return r;
+}
+
+// The maps `members` as in emit_members, with explicit rounding.
+void emit_members_rn(std::ostringstream& os, const GraphImpl& g, const std::vector<int>& members) {
+  std::map<int, Ex> ex;
+  auto val = [&](int v) {
+    auto it = ex.find(v);
+    Ex e;
+    if (it != ex.end()) e = it->second;
+    e.s = var(v);
+    return e;
+  };
+  for (int v : members) {
+    const Node& n = g.nodes[v];
+    const Ex a = n.in.empty() ? Ex() : val(n.in[0]);
+    const Ex b = n.in.size() > 1 ? val(n.in[1]) : Ex();
+    Ex e;
+    if (n.kind == Kind::Stencil) e.s = a.s;  // zero-step stencil: identity
+    else e = ex_op(n.op, n.dtype, n.imm, a, b);
+    e.uses = 0;
+    for (int m : members)
+      for (int o : g.nodes[m].in) e.uses += o == v;
+    os << "  const DCP_T " << var(v) << " = " << e.s << ";\n";
+    ex[v] = e;
+  }
+}
+
 void emit_members(std::ostringstream& os, const GraphImpl& g, const std::vector<int>& members) {
   for (int v : members) {
     const Node& n = g.nodes[v];
@@ -139,7 +219,6 @@ std::string red_op_fn(const GraphImpl& g, const std::vector<int>& reds) {
 // hand-written skeletons it includes, so the name (and the compiled-module
 // caches keyed by the source) changes exactly when one of them changes.
 uint64_t skeleton_hash(const std::string& body) {
-  std::string text = device_header_source();
   const std::pair<const char*, const char*> skel[] = {
       {"k_map.cuh", kernel_map_source()},
       {"k_stencil2d.cuh", kernel_stencil2d_source()},
@@ -149,9 +228,19 @@ uint64_t skeleton_hash(const std::string& body) {
       {"k_math64.cuh", kernel_math64_source()},
       {"k_stencil_adj.cuh", kernel_adj_source()},
       {"k_stencil2d_coop.cuh", kernel_coop_source()}};
-  for (const auto& k : skel)
-    if (body.find(std::string("#include \"") + k.first + "\"") != std::string::npos) text += k.second;
-  return fnv1a(text);
+  unsigned used = 0;
+  for (size_t i = 0; i < sizeof skel / sizeof skel[0]; ++i)
+    if (body.find(std::string("#include \"") + skel[i].first + "\"") != std::string::npos) used |= 1u << i;
+  // (the skeletons never change within a process: one hash per set of them)
+  static std::mutex mu;
+  static std::map<unsigned, uint64_t> known;
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = known.find(used);
+  if (it != known.end()) return it->second;
+  std::string text = device_header_source();
+  for (size_t i = 0; i < sizeof skel / sizeof skel[0]; ++i)
+    if (used >> i & 1u) text += skel[i].second;
+  return known[used] = fnv1a(text);
 }
 
 std::string finish(const std::string& prefix, const std::string& b) {
@@ -257,21 +346,8 @@ CodegenOut gen_axis_kernel(const GraphImpl& g, const Group& G, bool vec_ok) {
 
 namespace {
 
-// Functions shared by 2-D and 3-D stencil sources: input (prologue), post.
-void emit_stencil_io(std::ostringstream& os, const GraphImpl& g, const Group& G, bool first,
-                     bool last) {
-  os << "__device__ __forceinline__ DCP_T dcp_input(const DcpStParamsT<DCP_T>& p, const DCP_T* sc, "
-        "long long gi) {\n";
-  if (first && !G.members.empty()) {
-    for (size_t i = 0; i < G.loads.size(); ++i)
-      os << "  const DCP_T " << var(G.loads[i]) << " = p.ld[" << i << "][gi];\n";
-    for (size_t i = 0; i < G.scalars.size(); ++i)
-      os << "  const DCP_T " << var(G.scalars[i]) << " = sc[" << i << "];\n";
-    emit_members(os, g, G.members);
-    os << "  (void)sc;\n  return " << var(G.st_in) << ";\n}\n";
-  } else {
-    os << "  (void)sc;\n  return p.ld[0][gi];\n}\n";
-  }
+// Maps, stores and reductions after the last step.
+void emit_stencil_post(std::ostringstream& os, const GraphImpl& g, const Group& G, bool last) {
   os << "__device__ __forceinline__ void dcp_post(const DcpStParamsT<DCP_T>& p, const DCP_T* sc, "
         "long long gi, DCP_T v, DCP_T* st, DCP_T* rv) {\n";
   if (last) {
@@ -289,6 +365,23 @@ void emit_stencil_io(std::ostringstream& os, const GraphImpl& g, const Group& G,
   os << "  (void)p; (void)sc; (void)gi; (void)v; (void)st; (void)rv;\n}\n";
 }
 
+// Functions shared by 2-D and 3-D stencil sources: input (prologue), post.
+void emit_stencil_io(std::ostringstream& os, const GraphImpl& g, const Group& G, bool first,
+                     bool last) {
+  os << "__device__ __forceinline__ DCP_T dcp_input(const DcpStParamsT<DCP_T>& p, const DCP_T* sc, "
+        "long long gi) {\n";
+  if (first && !G.members.empty()) {
+    for (size_t i = 0; i < G.loads.size(); ++i)
+      os << "  const DCP_T " << var(G.loads[i]) << " = p.ld[" << i << "][gi];\n";
+    for (size_t i = 0; i < G.scalars.size(); ++i)
+      os << "  const DCP_T " << var(G.scalars[i]) << " = sc[" << i << "];\n";
+    emit_members_rn(os, g, G.members);
+    os << "  (void)sc;\n  return " << var(G.st_in) << ";\n}\n";
+  } else {
+    os << "  (void)sc;\n  return p.ld[0][gi];\n}\n";
+  }
+  emit_stencil_post(os, g, G, last);
+}
 // Deferred common weight of a linear run of binary64 stencil steps.  A step
 // u' = sum_k w_k u[p + o_k] whose weights are all exact multiples
 // w_k = f r_k of one weight f (r_k = 1 at f's own points) is computed as
@@ -475,24 +568,226 @@ void emit_term(std::ostringstream& os, int T, const std::string& a, const std::s
   else os << "  " << a << " = dcp_fma_rn(" << km.get(T, w) << ", " << x << ", " << a << ");\n";
 }
 
+// How every 1-D / 2-D kernel form evaluates one step's weighted sum, so that
+// all of them round alike.
+//
+// Row order (any stencil): the points sorted by row offset dy (ascending, the
+// listed order within a row), one multiply (or, on a deferred common weight,
+// a copy of a ratio-1 point) and fused multiply-adds.  A kernel that streams
+// rows then adds each arriving row to the sums of the rows it touches and
+// keeps 2 ry partial sums per column instead of 2 ry + 1 rows.
+//
+// Pair order (a 5-point star on a deferred weight whose four sides have ratio
+// 1): D(p) = w(west) + w(north) is also w(south) + w(east) of the cell one row
+// up and one column left, so
+//     sum(p) = (D(p) + r w(centre)) + D(p + (1, 1))
+// and a kernel that keeps D pays one add for two pairs of neighbours: 3
+// operations per cell instead of 4.  Steps that apply their weights keep the
+// row order: sums before the weights could leave the plain sum's range, and
+// weights before the sums round once more per point (measured: 1.3 times the
+// error of 50 binary32 steps).
+struct Sum2 {
+  Defer df;
+  bool pair = false;
+  double wc = 1.0;            // pair: the centre's ratio
+  std::vector<int> order;     // row order
+  std::vector<double> w;      // row order: weights (ratios) by point index
+};
+
+bool star_sides(const std::vector<int32_t>& offs, int npts, int& centre, int (&side)[4]) {
+  if (npts != 5) return false;
+  centre = -1;
+  for (int& v : side) v = -1;
+  for (int k = 0; k < npts; ++k) {
+    const int dz = offs[k * 3], dy = offs[k * 3 + 1], dx = offs[k * 3 + 2];
+    int* slot = dz ? nullptr
+                : dy == 0 && dx == 0 ? &centre
+                : dy == 0 && dx == -1 ? &side[0]   // west
+                : dy == -1 && dx == 0 ? &side[1]   // north
+                : dy == 0 && dx == 1 ? &side[2]    // east
+                : dy == 1 && dx == 0 ? &side[3] : nullptr;  // south
+    if (!slot || *slot >= 0) return false;
+    *slot = k;
+  }
+  return true;
+}
+
+// `offs`: the step's offsets (padded to 3 axes); `df`: its deferred weight.
+Sum2 plan_sum2(const std::vector<int32_t>& offs, const std::vector<double>& weights,
+               const Defer& df) {
+  Sum2 p;
+  p.df = df;
+  p.w = df.on ? df.ratio : weights;
+  const int n = (int)p.w.size();
+  int c, sd[4];
+  if (df.on && star_sides(offs, n, c, sd) && p.w[sd[0]] == 1.0 && p.w[sd[1]] == 1.0 &&
+      p.w[sd[2]] == 1.0 && p.w[sd[3]] == 1.0) {
+    p.pair = true;
+    p.wc = p.w[c];
+    return p;
+  }
+  for (int k = 0; k < n; ++k) p.order.push_back(k);
+  std::stable_sort(p.order.begin(), p.order.end(),
+                   [&](int a, int b) { return offs[a * 3 + 1] < offs[b * 3 + 1]; });
+  if (df.on)  // start from a ratio-1 point of the first row, which needs no multiply
+    for (int i = 1; i < n && offs[p.order[i] * 3 + 1] == offs[p.order[0] * 3 + 1]; ++i)
+      if (p.w[p.order[0]] != 1.0 && p.w[p.order[i]] == 1.0) {
+        std::rotate(p.order.begin(), p.order.begin() + i, p.order.begin() + i + 1);
+        break;
+      }
+  return p;
+}
+
+// x + y as the kernels of dtype T add: binary64 as a fused multiply-add by a
+// register of 1.0 (the same rounding at the pipe's full rate).
+std::string add_expr(int T, const std::string& x, const std::string& y, MulRegs& km) {
+  if (T == DCP_F64) return "dcp_fma_rn(" + x + ", " + km.get(T, 1.0) + ", " + y + ")";
+  return "dcp_add_rn(" + x + ", " + y + ")";
+}
+
+// One row-order term into accumulator a (`fresh`: the sum's first term).
+void emit_row_term(std::ostringstream& os, int T, const std::string& a, const std::string& from,
+                   const std::string& x, double w, bool fresh, bool deferred, MulRegs& km) {
+  os << "  " << a << " = ";
+  if (fresh && deferred && w == 1.0) os << x;
+  else if (fresh) os << "dcp_mul_rn(" << weight_literal(T, w) << ", " << x << ")";
+  else if (w == 1.0 && deferred) os << add_expr(T, x, from, km);
+  else os << "dcp_fma_rn(" << km.get(T, w) << ", " << x << ", " << from << ")";
+  os << ";\n";
+}
+
+// The whole sum of one cell as straight-line code declaring `acc`; x(dy, dx)
+// names the neighbour (kernels that hold a whole tile).
+template <class X>
+void emit_sum_cell(std::ostringstream& os, int T, const Sum2& p, const std::vector<int32_t>& offs,
+                   X x, MulRegs& km) {
+  os << "  DCP_T acc;\n";
+  if (p.pair) {
+    os << "  acc = " << add_expr(T, x(0, -1), x(-1, 0), km) << ";\n";
+    if (p.wc == 1.0) os << "  acc = " << add_expr(T, x(0, 0), "acc", km) << ";\n";
+    else os << "  acc = dcp_fma_rn(" << km.get(T, p.wc) << ", " << x(0, 0) << ", acc);\n";
+    os << "  const DCP_T d2 = " << add_expr(T, x(1, 0), x(0, 1), km) << ";\n";
+    os << "  acc = " << add_expr(T, "d2", "acc", km) << ";\n";
+  } else {
+    for (size_t i = 0; i < p.order.size(); ++i) {
+      const int k = p.order[i];
+      emit_row_term(os, T, "acc", "acc", x(offs[k * 3 + 1], offs[k * 3 + 2]), p.w[k], i == 0,
+                    p.df.on, km);
+    }
+  }
+  if (p.df.scale != 1.0)
+    os << "  acc = dcp_mul_rn(" << weight_literal(T, p.df.scale) << ", acc);\n";
+}
+
+// Unary / immediate maps applied in order to `v`.
+std::string epi_chain(const std::vector<std::pair<int, double>>& ops, int dtype) {
+  std::ostringstream os;
+  Ex cur;
+  cur.s = "v";
+  int k = 0;
+  for (const auto& o : ops) {
+    Ex e = ex_op(o.first, dtype, o.second, cur, Ex());
+    const std::string nv = "e" + std::to_string(k++);
+    os << "  const DCP_T " << nv << " = " << e.s << ";\n";
+    cur = e;
+    cur.s = nv;
+  }
+  os << "  return " << cur.s << ";\n";
+  return os.str();
+}
+
 // Epilogue chain of one step as a function of the weighted sum.
 std::string epi_body(const GraphImpl& g, const StepDesc& s) {
-  std::ostringstream os;
-  std::string cur = "v";
-  int k = 0;
-  for (int e : s.epi) {
-    std::string nv = "e" + std::to_string(k++);
-    os << "  const DCP_T " << nv << " = " << map_expr(g, e, cur, "") << ";\n";
-    cur = nv;
-  }
-  os << "  return " << cur << ";\n";
-  return os.str();
+  std::vector<std::pair<int, double>> ops;
+  for (int e : s.epi) ops.emplace_back(g.nodes[e].op, g.nodes[e].imm);
+  return epi_chain(ops, s.epi.empty() ? DCP_F64 : g.nodes[s.epi[0]].dtype);
 }
 
 }  // namespace
 
+// The arrival of one row in a level of the warp-stream kernel: dcp_row<S>
+// takes the row `a`, adds it to the level's partial sums `st` and gives the
+// finished row `out` (ry rows above `a`).  rm[k]: columns whose cells in
+// output row (row of a) - ry + k belong to a fixed ring (RINGM only).
+static void emit_stream_row(std::ostringstream& os, int T, int s, const Sum2& p,
+                            const std::vector<int32_t>& offs, int C, int ry, int rx, MulRegs& km) {
+  const int NST = 2 * ry;
+  os << "template <> struct DcpRow<" << s << "> {\n  template <bool RINGM>\n"
+     << "  static __device__ __forceinline__ void run(const DCP_T (&a)[" << C << "], DCP_T (&st)["
+     << (NST > 0 ? NST : 1) << "][" << C << "], DCP_T (&out)[" << C
+     << "], const DCP_T (&km)[DCP_NK], const unsigned (&rm)[" << ry + 1 << "]) {\n"
+     << "  (void)km; (void)st; (void)rm;\n";
+  if (p.df.on) os << "  // deferred common weight: the ratios w_k / f\n";
+  auto at = [](const char* n, int i) { return std::string(n) + "[" + std::to_string(i) + "]"; };
+  auto st = [](int k, int c) { return "st[" + std::to_string(k) + "][" + std::to_string(c) + "]"; };
+  if (p.pair) {
+    // (a deferred run has no fixed ring)
+    os << "  DCP_T d[" << C << "];\n  const DCP_T al = __shfl_up_sync(0xffffffffu, a[" << C - 1 << "], 1);\n";
+    for (int c = 0; c < C; ++c)
+      os << "  " << at("d", c) << " = " << add_expr(T, c ? at("a", c - 1) : "al", st(0, c), km) << ";\n";
+    os << "  const DCP_T dr = __shfl_down_sync(0xffffffffu, d[0], 1);\n";
+    for (int c = 0; c < C; ++c)
+      os << "  " << at("out", c) << " = " << add_expr(T, c + 1 < C ? at("d", c + 1) : "dr", st(1, c), km)
+         << ";\n";
+    for (int c = 0; c < C; ++c) {
+      if (p.wc == 1.0) os << "  " << st(1, c) << " = " << add_expr(T, at("a", c), at("d", c), km) << ";\n";
+      else os << "  " << st(1, c) << " = dcp_fma_rn(" << km.get(T, p.wc) << ", " << at("a", c) << ", "
+              << at("d", c) << ");\n";
+      os << "  " << st(0, c) << " = " << at("a", c) << ";\n";
+    }
+  } else {
+    bool left = false, right = false;
+    for (size_t k = 0; k < p.w.size(); ++k) {
+      left = left || offs[k * 3 + 2] < 0;
+      right = right || offs[k * 3 + 2] > 0;
+    }
+    if (left) {
+      os << "  DCP_T lf[" << rx << "];\n";
+      for (int q = 0; q < rx; ++q)
+        os << "  lf[" << rx - 1 - q << "] = __shfl_up_sync(0xffffffffu, a[" << C - 1 - q << "], 1);\n";
+    }
+    if (right) {
+      os << "  DCP_T rt[" << rx << "];\n";
+      for (int q = 0; q < rx; ++q)
+        os << "  rt[" << q << "] = __shfl_down_sync(0xffffffffu, a[" << q << "], 1);\n";
+    }
+    // stage k: output row (row of a) - ry + k receives its dy = ry - k points
+    for (int k = 0; k <= 2 * ry; ++k) {
+      const int dy = ry - k;
+      bool started = false;
+      std::vector<int> pts;
+      for (int i : p.order) {
+        if (offs[i * 3 + 1] < dy) started = true;
+        if (offs[i * 3 + 1] == dy) pts.push_back(i);
+      }
+      for (int c = 0; c < C; ++c) {
+        const std::string dst = k == 0 ? at("out", c) : st(k - 1, c);
+        const std::string src = k < 2 * ry ? st(k, c) : std::string("0");
+        bool fresh = !started;
+        const bool ring_sel = dy >= 0 && ry > 0;  // a ring cell's sum is its own value
+        os << "  {\n  DCP_T t = " << (started ? src : "(DCP_T)0") << ";\n";
+        for (int i : pts) {
+          const int cc = c + offs[i * 3 + 2];
+          const std::string x = cc < 0 ? at("lf", rx + cc) : (cc >= C ? at("rt", cc - C) : at("a", cc));
+          emit_row_term(os, T, "t", "t", x, p.w[i], fresh, p.df.on, km);
+          fresh = false;
+        }
+        if (ring_sel || ry == 0)
+          os << "  if (RINGM && ((rm[" << k << "] >> " << c << ") & 1u)) t = "
+             << (dy == 0 ? at("a", c) : src) << ";\n";
+        os << "  " << dst << " = t;\n  }\n";
+      }
+    }
+  }
+  if (p.df.scale != 1.0)
+    for (int c = 0; c < C; ++c)
+      os << "  " << at("out", c) << " = dcp_mul_rn(" << weight_literal(T, p.df.scale) << ", "
+         << at("out", c) << ");\n";
+  os << "  }\n};\n";
+}
+
 // Warp-stream form (k_stencil2d_stream.cuh) of a 1-D / 2-D stencil launch.
-static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, int s1) {
+static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, int s1, int max_vec) {
   NameScope names;
   const bool batch = G.kind == GroupKind::Batch;
   const int nd = batch ? 2 : (int)G.shape.size();
@@ -501,97 +796,86 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
   const bool first = s0 == 0, last = s1 == (int)G.steps.size();
   const int C = stream_cols_per_lane(T);
   const int ry = nd == 1 ? 0 : G.radius[1], rx = G.radius[2];
-  const int NR = 2 * ry + 1;
-  const int RXA = rx > 0 ? rx : 1;
+  const bool pro = !batch && first && !G.members.empty();
+  // elements per access: the widest that divides a row (batched: per instance)
+  int vec = 0;
+  if (!batch)
+    for (vec = std::min(C, max_vec); G.shape.back() % vec != 0;) vec /= 2;
   std::ostringstream os;
   os << "// dcp warp-stream stencil kernel: " << nsteps << " steps per launch, bc " << G.bc << ", "
      << nd << "-D" << (batch ? ", batched" : "") << "\n";
   os << "#define DCP_T " << dtype_cname(T) << "\n#define DCP_C " << C << "\n";
-  os << "#define DCP_THREADS " << G.threads << "\n#define DCP_BC " << G.bc << "\n";
+  // shared-memory ring: 8 rows (a window of 7 rows ahead hides device-memory
+  // latency from 4 warps per scheduler) per prefetch window and input array,
+  // 512 bytes each; fewer rows, then fewer warps per CTA where 192 KB is short
+  const int nload = pro ? (int)G.loads.size() : 1;
+  const int nin = std::max(1, nload);  // a prologue of broadcast scalars loads no array
+  int threads = G.threads, ring = 8 * G.prefetch;
+  auto smem = [&] { return threads / 32 * nin * ring * 512; };
+  while (smem() > 192 * 1024 && ring > 4) ring /= 2;
+  while (smem() > 192 * 1024 && threads > 32) threads = threads / 64 * 32;
+  os << "#define DCP_THREADS " << threads << "\n#define DCP_BC " << G.bc << "\n";
   os << "#define DCP_LAST " << (last ? 1 : 0) << "\n#define DCP_BATCH " << (batch ? 1 : 0) << "\n";
   os << "#define DCP_NSTORE " << (last ? (int)G.stores.size() : 1) << "\n#define DCP_NRED "
      << (last ? (int)G.reds.size() : 0) << "\n#define DCP_NSCALAR " << G.scalars.size() << "\n";
+  os << "#define DCP_NLOAD " << nload << "\n#define DCP_NIN " << nin << "\n#define DCP_PRO " << (pro ? 1 : 0)
+     << "\n#define DCP_POST "
+     << (last && (!G.post.empty() || !G.reds.empty() || G.stores.size() != 1) ? 1 : 0) << "\n";
   os << "#define DCP_RX " << rx << "\n#define DCP_RY " << ry << "\n#define DCP_NSTEPS " << nsteps
-     << "\n#define DCP_PDM " << G.prefetch << "\n";
+     << "\n#define DCP_R " << ring << "\n#define DCP_W " << stream_width(G, nsteps)
+     << "\n#define DCP_VEC " << vec << "\n";
   const Defer guard = first ? plan_defer(g, G, 0) : Defer();
   os << "#define DCP_GUARD " << (guard.on ? 1 : 0) << "\n";
   if (G.min_ctas > 0) os << "#define DCP_MINB " << G.min_ctas << "\n";
   os << red_op_fn(g, last ? G.reds : std::vector<int>{});
   os << "#include \"dcp_device.cuh\"\n";
-  if (!batch) emit_stencil_io(os, g, G, first, last);
-  std::ostringstream decls;  // declarations that need the multiplier count
-  decls << "template <int S> __device__ __forceinline__ void dcp_level(const DCP_T (&up)[" << NR
-        << "][" << C << "], const DCP_T (&lf)[" << NR << "][" << RXA << "], const DCP_T (&rt)["
-        << NR << "][" << RXA << "], DCP_T (&out)[" << C << "], const DCP_T (&km)[DCP_NK]);\n";
-  os << "template <int S> __device__ __forceinline__ DCP_T dcp_epi(DCP_T v);\n";
-  // which rows of each step read a neighbour column to the left / right
-  // (only those rows are exchanged between lanes)
-  std::vector<unsigned> lmask(nsteps, 0u), rmask(nsteps, 0u);
-  for (int s = 0; s < nsteps; ++s) {
-    const Node& sn = g.nodes[G.steps[s0 + s].node];
-    for (int k = 0; k < sn.npts(); ++k) {
-      const int row = ry + G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
-      if (dx < 0) lmask[s] |= 1u << row;
-      if (dx > 0) rmask[s] |= 1u << row;
+  if (!batch) {
+    // the prologue as a function of the loaded values (the kernel keeps raw
+    // loads in flight and evaluates the maps when the row arrives)
+    os << "__device__ __forceinline__ DCP_T dcp_pro(const DCP_T (&ld)[DCP_NIN], const DCP_T* sc) {\n"
+          "  (void)sc;\n";
+    if (pro) {
+      for (size_t i = 0; i < G.loads.size(); ++i)
+        os << "  const DCP_T " << var(G.loads[i]) << " = ld[" << i << "];\n";
+      for (size_t i = 0; i < G.scalars.size(); ++i)
+        os << "  const DCP_T " << var(G.scalars[i]) << " = sc[" << i << "];\n";
+      emit_members_rn(os, g, G.members);
+      os << "  return " << var(G.st_in) << ";\n}\n";
+    } else {
+      os << "  return ld[0];\n}\n";
     }
+    emit_stencil_post(os, g, G, last);
   }
-  auto mask_fn = [&](const char* name, const std::vector<unsigned>& m) {
-    os << "__device__ __forceinline__ constexpr bool " << name << "(int s, int d) {\n"
-       << "  constexpr unsigned m[" << nsteps << "] = {";
-    for (int s = 0; s < nsteps; ++s) os << (s ? ", " : "") << m[s] << "u";
-    os << "};\n  return (m[s] >> d) & 1u;\n}\n";
-  };
-  mask_fn("dcp_uses_lf", lmask);
-  mask_fn("dcp_uses_rt", rmask);
+  os << "template <int S> __device__ __forceinline__ DCP_T dcp_epi(DCP_T v);\n"
+     << "template <int S> struct DcpRow;\n";
   std::vector<double> scales;
   MulRegs km;
   km.on = T == DCP_F64;
   std::ostringstream sums;  // emitted after the multiplier table they use
   for (int s = 0; s < nsteps; ++s) {
-    std::ostringstream& os = sums;
     const StepDesc& sd = G.steps[s0 + s];
-    const Node& sn = g.nodes[sd.node];
-    os << "template <> __device__ __forceinline__ void dcp_level<" << s << ">(const DCP_T (&up)[" << NR
-       << "][" << C << "], const DCP_T (&lf)[" << NR << "][" << RXA << "], const DCP_T (&rt)[" << NR
-       << "][" << RXA << "], DCP_T (&out)[" << C << "], const DCP_T (&km)[DCP_NK]) {\n";
-    os << "  (void)lf; (void)rt; (void)km;\n";
-    const Defer df = plan_defer(g, G, s0 + s);
-    if (df.on) os << "  // deferred common weight: the ratios w_k / f\n";
-    scales.push_back(df.on ? df.scale : 0.0);
-    for (int c = 0; c < C; ++c) {
-      const std::string a = "a" + std::to_string(c);
-      for (int i = 0; i < sn.npts(); ++i) {
-        const int k = df.on ? df.order[i] : i;
-        int dy = G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
-        int cc = c + dx, row = ry + dy;
-        std::string x;
-        if (cc < 0) x = "lf[" + std::to_string(row) + "][" + std::to_string(rx + cc) + "]";
-        else if (cc >= C) x = "rt[" + std::to_string(row) + "][" + std::to_string(cc - C) + "]";
-        else x = "up[" + std::to_string(row) + "][" + std::to_string(cc) + "]";
-        emit_term(os, T, a, x, df.on ? df.ratio[k] : sn.weights[k], i == 0, df.on, km);
-      }
-      if (df.scale != 1.0) os << "  " << a << " = dcp_mul_rn(" << weight_literal(T, df.scale) << ", " << a << ");\n";
-      os << "  out[" << c << "] = " << a << ";\n";
-    }
-    os << "}\n";
-    os << "template <> __device__ __forceinline__ DCP_T dcp_epi<" << s << ">(DCP_T v) {\n"
-       << epi_body(g, sd) << "}\n";
+    const Sum2 p = plan_sum2(G.offsets, g.nodes[sd.node].weights, plan_defer(g, G, s0 + s));
+    scales.push_back(p.df.on ? p.df.scale : 0.0);
+    emit_stream_row(sums, T, s, p, G.offsets, C, ry, rx, km);
+    sums << "template <> __device__ __forceinline__ DCP_T dcp_epi<" << s << ">(DCP_T v) {\n"
+         << epi_body(g, sd) << "}\n";
   }
-  os << km.table() << decls.str() << sums.str();
+  os << km.table() << sums.str();
   os << "#include \"k_stencil2d_stream.cuh\"\n";
   CodegenOut out;
-  out.threads = G.threads;
-  out.smem_bytes = 0;
+  out.threads = threads;
+  out.smem_bytes = smem();
   for (double x : scales)
     if (x != 0.0) out.defer_scales = scales;
   out.guard_max_input = guard.on ? guard.max_input : 0.0;
+  out.vec = std::max(1, vec);
   out.source = finish(batch ? "dcp_bstream" : "dcp_stream", os.str());
   out.name = kname_of(out.source);
   return out;
 }
 
-CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1) {
-  if (G.variant == 1) return gen_stream_kernel(g, G, s0, s1);
+CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1, int max_vec) {
+  if (G.variant == 1) return gen_stream_kernel(g, G, s0, s1, max_vec);
   NameScope names;
   const bool batch = G.kind == GroupKind::Batch;
   const int nd = batch ? 2 : (int)G.shape.size();
@@ -643,17 +927,12 @@ CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1
       const Node& sn = g.nodes[sd.node];
       os << "template <> __device__ __forceinline__ DCP_T dcp_sum<" << s
          << ">(const DCP_T* A, int c, const DCP_T (&km)[DCP_NK]) {\n  (void)km;\n";
-      const Defer df = plan_defer(g, G, s0 + s);
-      if (df.on) os << "  // deferred common weight: the ratios w_k / f\n";
-      scales.push_back(df.on ? df.scale : 0.0);
-      for (int i = 0; i < sn.npts(); ++i) {
-        const int k = df.on ? df.order[i] : i;
-        int dy = G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
-        int off = dy * PW + dx;
-        std::string x = "A[c + (" + std::to_string(off) + ")]";
-        emit_term(os, T, "acc", x, df.on ? df.ratio[k] : sn.weights[k], i == 0, df.on, km);
-      }
-      if (df.scale != 1.0) os << "  acc = dcp_mul_rn(" << weight_literal(T, df.scale) << ", acc);\n";
+      const Sum2 p = plan_sum2(G.offsets, sn.weights, plan_defer(g, G, s0 + s));
+      if (p.df.on) os << "  // deferred common weight: the ratios w_k / f\n";
+      scales.push_back(p.df.on ? p.df.scale : 0.0);
+      emit_sum_cell(os, T, p, G.offsets, [&](int dy, int dx) {
+        return "A[c + (" + std::to_string(dy * PW + dx) + ")]";
+      }, km);
       os << "  return acc;\n}\n";
       os << "template <> __device__ __forceinline__ DCP_T dcp_epi<" << s << ">(DCP_T v) {\n"
          << epi_body(g, sd) << "}\n";
@@ -772,24 +1051,25 @@ int vjp_reads(int op) {
 
 // Cotangent of the operand of op from the cotangent a of its result (the
 // same expressions as the per-op reverse maps of the adjoint builder).
-std::string vjp_expr(int op, double imm, int T, const std::string& a, const std::string& X,
-                     const std::string& Y) {
+std::string vjp_expr(int op, double imm, int T, const std::string& as, const std::string& Xs,
+                     const std::string& Ys) {
+  Ex a, X, Y;
+  a.s = as;
+  X.s = Xs;
+  Y.s = Ys;
+  auto e = [&](int o, double i, const Ex& p, const Ex& q = Ex()) { return ex_op(o, T, i, p, q); };
   switch (op) {
-    case DCP_NEG: return op_expr(DCP_NEG, T, 0, a, "");
-    case DCP_ABS: return op_expr(DCP_MUL, T, 0, op_expr(kOpSign, T, 0, X, ""), a);
-    case DCP_EXP: return op_expr(DCP_MUL, T, 0, Y, a);
-    case DCP_SIN: return op_expr(DCP_MUL, T, 0, op_expr(DCP_COS, T, 0, X, ""), a);
-    case DCP_COS:
-      return op_expr(DCP_MUL, T, 0, op_expr(DCP_NEG, T, 0, op_expr(DCP_SIN, T, 0, X, ""), ""), a);
-    case DCP_TANH:
-      return op_expr(DCP_MUL, T, 0,
-                     op_expr(DCP_RSUB_S, T, 1.0, op_expr(DCP_SQUARE, T, 0, Y, ""), ""), a);
-    case DCP_SQRT: return op_expr(DCP_DIV, T, 0, op_expr(DCP_MUL_S, T, 0.5, a, ""), Y);
-    case DCP_SQUARE:
-      return op_expr(DCP_MUL, T, 0, op_expr(DCP_MUL_S, T, 2.0, X, ""), a);
-    case DCP_ADD_S: case DCP_SUB_S: return a;
-    case DCP_MUL_S: return op_expr(DCP_MUL_S, T, imm, a, "");
-    case DCP_RSUB_S: return op_expr(DCP_NEG, T, 0, a, "");
+    case DCP_NEG: return e(DCP_NEG, 0, a).s;
+    case DCP_ABS: return e(DCP_MUL, 0, e(kOpSign, 0, X), a).s;
+    case DCP_EXP: return e(DCP_MUL, 0, Y, a).s;
+    case DCP_SIN: return e(DCP_MUL, 0, e(DCP_COS, 0, X), a).s;
+    case DCP_COS: return e(DCP_MUL, 0, e(DCP_NEG, 0, e(DCP_SIN, 0, X)), a).s;
+    case DCP_TANH: return e(DCP_MUL, 0, e(DCP_RSUB_S, 1.0, e(DCP_SQUARE, 0, Y)), a).s;
+    case DCP_SQRT: return e(DCP_DIV, 0, e(DCP_MUL_S, 0.5, a), Y).s;
+    case DCP_SQUARE: return e(DCP_MUL, 0, e(DCP_MUL_S, 2.0, X), a).s;
+    case DCP_ADD_S: case DCP_SUB_S: return as;
+    case DCP_MUL_S: return e(DCP_MUL_S, imm, a).s;
+    case DCP_RSUB_S: return e(DCP_NEG, 0, a).s;
   }
   fail(DCP_E_UNSUPPORTED, std::string("adjoint: no reverse rule for epilogue op ") + op_name(op));
 }
@@ -830,48 +1110,40 @@ CodegenOut gen_adj_kernel(const GraphImpl& g, const Group& G) {
   std::ostringstream fn;  // emitted after the multiplier table they use
   for (int s = 0; s < K; ++s) {
     const AdjStep& st = n.chain[s];
-    const int P = (int)st.weights.size();
     for (int dir = 0; dir < 2; ++dir) {  // 0: forward sum, 1: transposed sum
       fn << "template <> __device__ __forceinline__ DCP_T " << (dir ? "dcp_bsum<" : "dcp_fsum<") << s
          << ">(const DCP_T* A, int c, const DCP_T (&km)[DCP_NK]) {\n  (void)km;\n";
-      for (int k = 0; k < P; ++k) {
-        const int sg = dir ? -1 : 1;
-        const int dy = sg * G.offsets[k * 3 + 1], dx = sg * G.offsets[k * 3 + 2];
-        emit_term(fn, T, "acc", "A[c + (" + std::to_string(dy * PW + dx) + ")]", st.weights[k],
-                  k == 0, false, km);
-      }
+      std::vector<int32_t> offs = G.offsets;  // transposed: negated offsets
+      if (dir)
+        for (auto& o : offs) o = -o;
+      emit_sum_cell(fn, T, plan_sum2(offs, st.weights, Defer()), offs, [&](int dy, int dx) {
+        return "A[c + (" + std::to_string(dy * PW + dx) + ")]";
+      }, km);
       fn << "  return acc;\n}\n";
     }
     // forward epilogue
     fn << "template <> __device__ __forceinline__ DCP_T dcp_fepi<" << s << ">(DCP_T v) {\n";
-    std::string cur = "v";
-    for (size_t j = 0; j < st.epi.size(); ++j) {
-      std::string nv = "e" + std::to_string(j);
-      fn << "  const DCP_T " << nv << " = " << op_expr(st.epi[j].first, T, st.epi[j].second, cur, "")
-         << ";\n";
-      cur = nv;
-    }
-    fn << "  return " << cur << ";\n}\n";
+    fn << epi_chain(st.epi, T) << "}\n";
     // reverse of the epilogue: intermediates recomputed from z when read
     fn << "template <> __device__ __forceinline__ DCP_T dcp_vjp<" << s
        << ">(DCP_T g, DCP_T z, DCP_T u) {\n  (void)z; (void)u;\n";
     const int m = (int)st.epi.size();
-    std::vector<std::string> val(m + 1);  // val[0] = z, val[j] = result of op j-1
-    val[0] = "z";
+    std::vector<Ex> val(m + 1);  // val[0] = z, val[j] = result of op j-1
+    val[0].s = "z";
     const bool need = adj_needs_z(st.epi);
     for (int j = 0; j < m; ++j) {
       if (need && j + 1 < m) {
-        val[j + 1] = "f" + std::to_string(j);
-        fn << "  const DCP_T " << val[j + 1] << " = "
-           << op_expr(st.epi[j].first, T, st.epi[j].second, val[j], "") << ";\n";
+        val[j + 1] = ex_op(st.epi[j].first, T, st.epi[j].second, val[j], Ex());
+        fn << "  const DCP_T f" << j << " = " << val[j + 1].s << ";\n";
+        val[j + 1].s = "f" + std::to_string(j);
       }
     }
-    if (m > 0) val[m] = "u";
+    if (m > 0) val[m] = Ex(), val[m].s = "u";
     std::string a = "g";
     for (int j = m - 1; j >= 0; --j) {
       std::string nv = "a" + std::to_string(j);
       fn << "  const DCP_T " << nv << " = "
-         << vjp_expr(st.epi[j].first, st.epi[j].second, T, a, val[j], val[j + 1]) << ";\n";
+         << vjp_expr(st.epi[j].first, st.epi[j].second, T, a, val[j].s, val[j + 1].s) << ";\n";
       a = nv;
     }
     fn << "  return " << a << ";\n}\n";

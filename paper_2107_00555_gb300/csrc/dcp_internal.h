@@ -243,7 +243,7 @@ struct CodegenOut {
   std::string source;
   int smem_bytes = 0;
   int threads = 256;
-  int vec = 1;     // axis reductions: elements per load
+  int vec = 1;     // axis reductions, warp-stream stencils: elements per access
   int axmode = 0;  // axis reductions: 0 vectors along inner, 1 along the reduced axis
   // stencil launches: per step, the factor applied after the step when it
   // sums ratios to a deferred common weight (1: none), 0 for a plain sum;
@@ -255,7 +255,10 @@ struct CodegenOut {
 };
 CodegenOut gen_map_kernel(const GraphImpl& g, const Group& grp, bool vec_ok);
 // Stencil launch `chunk` covers steps [s0, s1) of the group.
-CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& grp, int s0, int s1);
+// (warp stream: max_vec bounds the elements per access, for buffers off a
+// 16-byte boundary).
+CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& grp, int s0, int s1,
+                              int max_vec = 16);
 CodegenOut gen_batch_kernel(const GraphImpl& g, const Group& grp, int s0, int s1);
 CodegenOut gen_axis_kernel(const GraphImpl& g, const Group& grp, bool vec_ok);
 // reverse of a chunk of a 1-D / 2-D stencil chain, forward recomputed in the tile
@@ -273,8 +276,12 @@ constexpr int kMaxIO = 16;       // loads / stores / reductions per kernel
 
 // Warp-stream stencil geometry: columns per lane and columns written per warp.
 inline int stream_cols_per_lane(int dtype) { return dtype == DCP_F64 || dtype == DCP_I64 ? 2 : 4; }
-inline int stream_width(const Group& G) {
-  return 32 * stream_cols_per_lane(G.dtype) - 2 * G.depth * G.radius[2];
+// Columns a warp writes per row in a launch of nsteps steps: the strip minus
+// its halos, the left one rounded up and the width rounded down to whole
+// vectors, so that strips start on vector boundaries of an aligned row.
+inline int stream_width(const Group& G, int nsteps) {
+  const int C = stream_cols_per_lane(G.dtype), h = nsteps * G.radius[2];
+  return (32 * C - (h + C - 1) / C * C - h) / C * C;
 }
 bool stream_eligible(const Group& G, int depth);
 // can the cooperative form run this group with a ty x tx tile (steps <= 63,

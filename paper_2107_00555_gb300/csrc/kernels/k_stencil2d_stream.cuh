@@ -1,31 +1,51 @@
 // k_stencil2d_stream.cuh -- register-resident, warp-streamed time tiling of
-// a 1-D / 2-D iterated stencil (zero or fixed-ring boundary).
+// a 1-D / 2-D iterated stencil (any boundary rule).
 //
-// A warp owns a strip of 32*C consecutive columns (C per lane) and streams
-// down the rows of its strip.  The DCP_NSTEPS steps of one launch are kept as
-// a pipeline of time levels in registers: when input row j arrives (level 0),
-// level l computes row j - l*RY from the 2*RY+1 most recent rows of level
-// l-1, so each row passes through all levels while it is in registers.
-// Neighbours along x come from the adjacent lanes by warp shuffles; the strip
-// loses RX columns of validity per level at each edge, so a warp writes
-// W = 32*C - 2*NSTEPS*RX columns.  There is no shared memory and no barrier
-// inside the stream; device memory is read once (plus the strip overlap) and
-// written once per NSTEPS steps.
+// A warp owns a strip of 32*C consecutive columns (C per lane, one 16-byte
+// vector) and streams down the rows of its strip.  The DCP_NSTEPS steps of
+// one launch are a pipeline of time levels in registers: when row j of the
+// input arrives, level l finishes row j - l*RY.  A level keeps no rows: an
+// arriving row is added at once to the 2*RY partial sums per column that it
+// touches (DcpRow, generated), so a level's state is 2*RY values per column
+// and each row costs its sums plus two lane exchanges.  Device memory is read
+// once (plus the strip overlap) and written once per DCP_NSTEPS steps.
+//
+// Input rows reach the warp through a ring of DCP_R rows in shared memory that
+// belongs to it alone, filled by asynchronous copies DCP_R - 1 rows ahead: no
+// block barrier, no register and no scoreboard is held by a load in flight.
+// (Rows prefetched into registers instead left each row waiting for about one
+// memory latency, 0.75 us whatever the number of levels: a warp has six
+// scoreboards, and the lane exchanges need them too.)
+//
+// Measured on a GB300 against the form that kept 2*RY + 1 rows per level and
+// read them element by element: 4000 x 4100 binary32, fixed ring, 50 steps, 4
+// per launch 526 -> 369 us; 2047 x 2051 binary64, periodic, 20 steps, 2 per
+// launch 722 (shared-memory tiles) -> 594 us; the 20-step reverse pass of a
+// 4096^2 binary32 chain with its loss, one step per launch, 3.01 -> 1.79 ms.
 //
 // Work items are (array, strip, row segment); a segment streams its rows plus
-// NSTEPS*RY warm-up rows above it.  Warps stride through the items (items of
-// the largest arrays first in batched launches).
+// NSTEPS*RY warm-up rows above and below it.  Warps stride through the items
+// (items of the largest arrays first in batched launches).  A strip writes
+// DCP_W columns starting at a multiple of C, its first lane HX (the halo
+// rounded up to whole vectors) columns to the left, so that rows of a 16-byte
+// multiple are read and written in whole vectors; other row lengths fall back
+// to the widest access that divides them.
+//
+// Boundaries: ZERO clears the columns (CHECK strips) and rows outside the
+// array at every level; FIXED_RING lets the sums of ring cells carry the
+// cell's own value; PERIODIC reads rows and columns at their wrapped
+// positions and computes the copies like the cells they copy.
+//
+// Bound: instruction issue (binary32) or the FP64 pipe (binary64).  Per level
+// and row a 5-point binary32 step issues 20 arithmetic instructions and 2
+// shuffles for 128 columns.
 //
 // The generated prefix defines DCP_T, DCP_C, DCP_RX, DCP_RY, DCP_NSTEPS,
-// DCP_BC, DCP_THREADS, DCP_KNAME, DCP_BATCH, DCP_LAST, DCP_PDM, DCP_GUARD, DCP_MINB,
-// DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
-//   T    dcp_input(const DcpStParams& p, const T* sc, long long i)   (prologue)
-//   void dcp_level<L>(const T (&up)[NR][C], const T (&lf)[NR][RX], const T (&rt)[NR][RX],
-//                     T (&out)[C], const T (&km)[DCP_NK])   weighted sum of step L
-//                     (rows up[RY+dy]; km: its multipliers, see dcp_load_multipliers),
+// DCP_BC, DCP_THREADS, DCP_KNAME, DCP_BATCH, DCP_LAST, DCP_R, DCP_GUARD, DCP_MINB,
+// DCP_W, DCP_VEC (elements per access, 0: per instance), DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions after the last step), DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
+//   T    dcp_pro(const T (&ld)[DCP_NIN], const T* sc)     input maps on the loaded values
+//   struct DcpRow<L>::run<RINGM>(a, st, out, km, rm)      arrival of row a in level L+1
 //   T    dcp_epi<L>(T v)                 epilogue maps fused after step L
-//   bool dcp_uses_lf(int L, int d), dcp_uses_rt(int L, int d)   (constexpr)
-//        whether step L reads a left / right neighbour column in row d
 //   void dcp_post(const DcpStParams& p, const T* sc, long long i, T v, T* st, T* rv)
 typedef DCP_T T;
 typedef typename DcpFin<T>::type F;
@@ -38,268 +58,301 @@ typedef typename DcpFin<T>::type F;
 #define DCP_BC_PERIODIC 1
 #define DCP_BC_FIXED_RING 2
 
-constexpr int NR = 2 * DCP_RY + 1;                 // rows kept per level
 constexpr int K = DCP_NSTEPS;
 constexpr int C = DCP_C;
+constexpr int RY = DCP_RY;
+constexpr int NST = DCP_ARR(2 * RY);               // partial sums per column and level
 constexpr int SPAN = 32 * C;                       // columns held by a warp
-constexpr int W = SPAN - 2 * K * DCP_RX;           // columns written by a warp
-static_assert(W > 0, "strip too narrow for the number of steps");
-constexpr int RXA = DCP_RX > 0 ? DCP_RX : 1;
+constexpr int HX = (K * DCP_RX + C - 1) / C * C;   // left halo, whole vectors
+constexpr int W = DCP_W;                           // columns written by a warp
+static_assert(W > 0 && W % C == 0 && HX + W + K * DCP_RX <= SPAN,
+              "strip too narrow for the number of steps");
+constexpr int RING = DCP_BC == DCP_BC_FIXED_RING ? RY : 0;  // ring rows
+
+constexpr int R = DCP_R;                           // rows of a warp's ring
+constexpr int D = R - 1;                           // rows requested ahead
+constexpr int ROWB = SPAN * (int)sizeof(T);        // bytes of a row
+static_assert(R >= 2, "the ring holds the current row and at least one ahead");
 
 typedef DcpStParamsT<T> DcpStParams;
 
-__device__ __forceinline__ constexpr int dcp_mod(int a, int m) { return ((a % m) + m) % m; }
+__device__ __forceinline__ int dcp_wrap(int q, int n) {
+  if ((unsigned)q < (unsigned)n) return q;
+  int r = q % n;
+  return r < 0 ? r + n : r;
+}
+
+// V consecutive elements as one access.
+template <int V> struct DcpAcc;
+template <> struct DcpAcc<1> { typedef T type; };
+template <> struct DcpAcc<2> { typedef typename DcpVec2<T>::type type; };
+template <> struct DcpAcc<4> { typedef uint4 type; };  // C = 4: binary32
+
+// Asynchronous copy of V elements into the ring (zeros when !ok).
+template <int V>
+__device__ __forceinline__ void dcp_copy(unsigned dst, const T* src, bool ok) {
+  constexpr int B = V * (int)sizeof(T);
+  const int n = ok ? B : 0;
+  if constexpr (B == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(B), "r"(n) : "memory");
+}
+__device__ __forceinline__ void dcp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void dcp_wait_copies() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // One array (or instance) and the part of it a work item covers.
 struct DcpItem {
-  const T* in;   // batched: instance input; single: unused (dcp_input reads p.ld)
-  T* out;        // batched: instance output
+  const T* in[DCP_NIN];
   int ny, nx;
   int x0;        // first written column
   int y0, y1;    // rows written
+  int vec;       // batched: elements per access (C: 16-byte rows, else 2 or 1)
 };
 
-// The lane's columns in a work item: the first one, and per column a bit
-// mask that keeps a value (all ones: the column lies inside the array) or
-// clears it to +0 (outside), computed once per item.
+// The lane's columns in a work item.
 struct DcpCols {
   int col0;
-  typename DcpBits<T>::type keep[C];
-  T km[DCP_NK];  // multipliers of the sums (see dcp_load_multipliers)
+  unsigned ring;                       // bit c: the column belongs to a fixed ring
+  typename DcpBits<T>::type keep[C];   // all ones inside the array, else 0
+  // copies: access i of the lane covers columns lane + 32 i of the strip in
+  // units of V elements, so that a warp's copies are contiguous
+  int pcol[C];                         // periodic CHECK strips: the wrapped column of access i (V = 1)
+  unsigned dst;                        // shared address of the warp's ring
 };
 
 // CHECK: the strip reaches outside the array (per-column tests).  ROWS: every
-// row touched by this iteration lies inside the array and outside a fixed
-// ring (no row tests).
-template <int L, int P, bool CHECK, bool ROWS>
-__device__ __forceinline__ void dcp_level_step(T (&ring)[K > 1 ? K : 1][NR][C], int j,
-                                               const DcpItem& it, const DcpCols& cols,
-                                               T (&outv)[C],
-                                               bool& out_ok) {
-  // level L (1-based) computes row y = j - L*RY from level L-1
-  constexpr int l = L - 1;  // source level
-  const int y = j - L * DCP_RY;
-  T up[NR][C];
+// row this iteration touches lies inside the array and outside a fixed ring.
+template <int L, bool CHECK, bool ROWS>
+__device__ __forceinline__ void dcp_levels(T (&a)[C], T (&st)[K][NST][C], int j, const DcpItem& it,
+                                           const DcpCols& cols, const T (&km)[DCP_NK]) {
+  if constexpr (L < K) {
+    constexpr bool RINGM = DCP_BC == DCP_BC_FIXED_RING && (CHECK || !ROWS);
+    const int y = j - (L + 1) * RY;  // the row this level finishes
+    unsigned rm[RY + 1];
 #pragma unroll
-  for (int d = 0; d < NR; ++d)
-#pragma unroll
-    for (int c = 0; c < C; ++c) up[d][c] = ring[l][dcp_mod(P - L * DCP_RY + d - DCP_RY, NR)][c];
-  // neighbour columns from the adjacent lanes, only for the rows the step
-  // reads off-centre
-  T lf[NR][RXA], rt[NR][RXA];
-#pragma unroll
-  for (int d = 0; d < NR; ++d)
-#pragma unroll
-    for (int q = 0; q < RXA; ++q) lf[d][q] = rt[d][q] = (T)0;
-#pragma unroll
-  for (int d = 0; d < NR; ++d)
-#pragma unroll
-    for (int q = 0; q < DCP_RX; ++q) {
-      if (dcp_uses_lf(L - 1, d))
-        lf[d][DCP_RX - 1 - q] = __shfl_up_sync(0xffffffffu, up[d][C - 1 - q], 1);
-      if (dcp_uses_rt(L - 1, d)) rt[d][q] = __shfl_down_sync(0xffffffffu, up[d][q], 1);
+    for (int k = 0; k <= RY; ++k) {
+      rm[k] = 0u;
+      if (RINGM) {
+        const bool rr = !ROWS && (y + k < RY || y + k >= it.ny - RY);
+        rm[k] = rr ? ~0u : cols.ring;
+      }
     }
-  T v[C];
-  dcp_level<L - 1>(up, lf, rt, v, cols.km);
-  const bool row_in = ROWS || (unsigned)y < (unsigned)it.ny;
-  if (!CHECK) {
-    // every column of the strip lies inside the array (and outside a fixed
-    // ring): only the row, uniform across the warp, needs a test
-    const bool ring_row =
-        !ROWS && DCP_BC == DCP_BC_FIXED_RING && (y < DCP_RY || y >= it.ny - DCP_RY);
-    if (!row_in) {
+    T v[C];
+    DcpRow<L>::template run<RINGM>(a, st[L], v, km, rm);
 #pragma unroll
-      for (int c = 0; c < C; ++c) v[c] = (T)0;
-    } else if (ring_row) {
+    for (int c = 0; c < C; ++c) v[c] = dcp_epi<L>(v[c]);
+    if (DCP_BC == DCP_BC_ZERO) {
+      // ghost zeros at every level, exact for any value an epilogue leaves
+      // there (a bitwise AND, NaN included)
+      if (!ROWS && (unsigned)y >= (unsigned)it.ny) {
 #pragma unroll
-      for (int c = 0; c < C; ++c) v[c] = dcp_epi<L - 1>(up[DCP_RY][c]);
+        for (int c = 0; c < C; ++c) v[c] = (T)0;
+      } else if (CHECK) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) v[c] = dcp_keep(v[c], cols.keep[c]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) a[c] = v[c];
+    dcp_levels<L + 1, CHECK, ROWS>(a, st, j, it, cols, km);
+  }
+}
+
+template <int V>
+__device__ __forceinline__ void dcp_st_row(T* p, const T (&src)[C], unsigned in) {
+  typedef typename DcpAcc<V>::type A;
+#pragma unroll
+  for (int u = 0; u < C / V; ++u) {
+    union { A a; T t[V]; } x;
+#pragma unroll
+    for (int v = 0; v < V; ++v) x.t[v] = src[u * V + v];
+    if ((in >> (u * V)) & 1u) *reinterpret_cast<A*>(p + u * V) = x.a;
+  }
+}
+
+// Requests a row (V elements per copy) from p, the strip's first column.
+template <int V, bool CHECK>
+__device__ __forceinline__ void dcp_fetch_units(unsigned dst, const T* row, int first, int nx,
+                                                bool row_ok) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < C / V; ++i) {
+    const int e = (lane + 32 * i) * V;
+    const bool ok = row_ok && (!CHECK || (unsigned)(first + e) < (unsigned)nx);
+    dcp_copy<V>(dst + e * (int)sizeof(T), ok ? row + first + e : row, ok);
+  }
+}
+
+// Requests input row j into ring slot `slot` (zeros outside the array).
+template <bool CHECK, bool ROWS>
+__device__ __forceinline__ void dcp_fetch_row(int slot, int j, const DcpItem& it,
+                                              const DcpCols& cols) {
+  const bool row_ok = ROWS || DCP_BC == DCP_BC_PERIODIC || (unsigned)j < (unsigned)it.ny;
+  const int row = ROWS ? j : (DCP_BC == DCP_BC_PERIODIC ? dcp_wrap(j, it.ny) : (row_ok ? j : 0));
+  const int first = it.x0 - HX;
+#pragma unroll
+  for (int l = 0; l < DCP_NLOAD; ++l) {
+    const T* p = it.in[l] + (long long)row * it.nx;
+    const unsigned dst = cols.dst + (l * R + slot) * ROWB;
+    const int vec = DCP_VEC > 0 ? DCP_VEC : it.vec;
+    if (DCP_BC == DCP_BC_PERIODIC && CHECK) {
+#pragma unroll
+      for (int i = 0; i < C; ++i)
+        dcp_copy<1>(dst + ((threadIdx.x & 31) + 32 * i) * (int)sizeof(T), p + cols.pcol[i], true);
+    } else if (vec == C) {
+      dcp_fetch_units<C, CHECK>(dst, p, first, it.nx, row_ok);
+    } else if (C > 2 && vec == 2) {
+      dcp_fetch_units<2, CHECK>(dst, p, first, it.nx, row_ok);
     } else {
-#pragma unroll
-      for (int c = 0; c < C; ++c) v[c] = dcp_epi<L - 1>(v[c]);
+      dcp_fetch_units<1, CHECK>(dst, p, first, it.nx, row_ok);
     }
-  } else if (DCP_BC == DCP_BC_ZERO) {
-    // columns outside the array read as ghost zeros at every level: the
-    // item's bit masks clear them (one bitwise AND per column, and exact for
-    // any value the epilogue leaves there, NaN included)
-    if (!row_in) {
+  }
+  dcp_commit();
+}
+
+__device__ __forceinline__ int dcp_next_slot(int s) { return s + 1 == R ? 0 : s + 1; }
+
+// One stream iteration: input row j from ring slot `slot`; row j + D is
+// requested into the slot that row j - 1 has left.
+template <bool CHECK, bool ROWS, class Pro, class Output>
+__device__ __forceinline__ void dcp_iter(T (&st)[K][NST][C], int& slot, int j, const DcpItem& it,
+                                         const DcpCols& cols, const T (&km)[DCP_NK], Pro& pro,
+                                         Output& output, DcpGuard& guard) {
+  dcp_wait_copies<D - 1>();  // this lane's copies of row j have landed
+  __syncwarp();              // every lane's have, and row j - 1 has been read
+  T a[C];
+  {
+    union { uint4 v; T t[C]; } x[DCP_NIN];
+    if (DCP_NLOAD == 0) x[0].v = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int c = 0; c < C; ++c) v[c] = (T)0;
-    } else {
-#pragma unroll
-      for (int c = 0; c < C; ++c) v[c] = dcp_keep(dcp_epi<L - 1>(v[c]), cols.keep[c]);
-    }
-  } else {
+    for (int l = 0; l < DCP_NLOAD; ++l)
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(x[l].v.x), "=r"(x[l].v.y), "=r"(x[l].v.z), "=r"(x[l].v.w)
+                   : "r"(cols.dst + (l * R + slot) * ROWB + (threadIdx.x & 31) * 16)
+                   : "memory");
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      const int col = cols.col0 + c;
-      const bool in = row_in && (unsigned)col < (unsigned)it.nx;
-      T r;
-      if (!in) {
-        r = (T)0;
-      } else if (DCP_BC == DCP_BC_FIXED_RING &&
-                 ((!ROWS && (y < DCP_RY || y >= it.ny - DCP_RY)) || col < DCP_RX ||
-                  col >= it.nx - DCP_RX)) {
-        r = dcp_epi<L - 1>(up[DCP_RY][c]);  // ring cell keeps its value; epilogue still applies
-      } else {
-        r = dcp_epi<L - 1>(v[c]);
-      }
-      v[c] = r;
+      T ld[DCP_NIN];
+#pragma unroll
+      for (int l = 0; l < DCP_NIN; ++l) ld[l] = x[l].t[c];
+      a[c] = pro(ld);
     }
   }
-  if constexpr (L < K) {
+  if (DCP_PRO && DCP_BC != DCP_BC_PERIODIC) {
+    // the maps of the zeros read outside the array need not be 0
+    if (!ROWS && (unsigned)j >= (unsigned)it.ny) {
 #pragma unroll
-    for (int c = 0; c < C; ++c) ring[L][dcp_mod(P - L * DCP_RY, NR)][c] = v[c];
-  } else {
+      for (int c = 0; c < C; ++c) a[c] = (T)0;
+    } else if (CHECK) {
 #pragma unroll
-    for (int c = 0; c < C; ++c) outv[c] = v[c];
-    out_ok = row_in;
+      for (int c = 0; c < C; ++c) a[c] = dcp_keep(a[c], cols.keep[c]);
+    }
   }
-}
-
-template <int L, int P, bool CHECK, bool ROWS>
-__device__ __forceinline__ void dcp_levels(T (&ring)[K > 1 ? K : 1][NR][C], int j,
-                                           const DcpItem& it, const DcpCols& cols,
-                                           T (&outv)[C],
-                                           bool& out_ok) {
-  if constexpr (L <= K) {
-    dcp_level_step<L, P, CHECK, ROWS>(ring, j, it, cols, outv, out_ok);
-    dcp_levels<L + 1, P, CHECK, ROWS>(ring, j, it, cols, outv, out_ok);
-  }
-}
-
-// Input rows in flight.  Row j lives in queue slot j mod PD and in ring slot
-// j mod NR; PD is a multiple of NR and iterations are unrolled by PD, so both
-// are compile-time constants and no register holding an outstanding load is
-// ever moved.  DCP_PDM row windows are requested ahead.
-constexpr int PD = NR * (NR > 1 ? DCP_PDM : 2 * DCP_PDM);
-
-template <bool CHECK, bool ROWS, class Input>
-__device__ __forceinline__ void dcp_fetch_row(T (&dst)[C], int j, const DcpItem& it,
-                                              const DcpCols& cols,
-                                              Input& input) {
-  const long long base = (long long)j * it.nx + cols.col0;
-  const bool row_ok = ROWS || (unsigned)j < (unsigned)it.ny;
+  if (DCP_GUARD) {
 #pragma unroll
-  for (int c = 0; c < C; ++c) {
-    const bool ok = row_ok && (!CHECK || (unsigned)(cols.col0 + c) < (unsigned)it.nx);
-    dst[c] = ok ? input(base + c) : (T)0;
+    for (int c = 0; c < C; ++c) guard.see(a[c]);
   }
+  dcp_fetch_row<CHECK, ROWS>(slot == 0 ? R - 1 : slot - 1, j + D, it, cols);
+  slot = dcp_next_slot(slot);
+  dcp_levels<0, CHECK, ROWS>(a, st, j, it, cols, km);
+  const int y = j - K * RY;
+  if (y >= it.y0 && y < it.y1) output(y, a);
 }
 
-// One stream iteration: input row j, P = j mod PD.  Row j + PD is requested
-// into the slot row j vacates before the levels are computed, so its load
-// latency overlaps PD iterations of arithmetic.
-template <int P, bool CHECK, bool ROWS, class Input, class Output>
-__device__ __forceinline__ void dcp_iter(T (&ring)[K > 1 ? K : 1][NR][C], T (&q)[PD][C], int j,
-                                         const DcpItem& it, const DcpCols& cols, Input& input,
-                                         Output& output, DcpGuard& guard) {
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    ring[0][P % NR][c] = q[P][c];
-    if (DCP_GUARD) guard.see(q[P][c]);  // arrived: requested PD iterations ago
-  }
-  dcp_fetch_row<CHECK, ROWS>(q[P], j + PD, it, cols, input);
-  T outv[C];
-  bool out_ok = false;
-  dcp_levels<1, P % NR, CHECK, ROWS>(ring, j, it, cols, outv, out_ok);
-  const int y = j - K * DCP_RY;
-  if (ROWS || (out_ok && y >= it.y0 && y < it.y1)) output(y, outv);
-}
-
-// Iterations j .. j + (PD - P) - 1 with phases P .. PD-1.
-template <int P, bool CHECK, bool ROWS, class Input, class Output>
-__device__ __forceinline__ void dcp_iters(T (&ring)[K > 1 ? K : 1][NR][C], T (&q)[PD][C], int j,
-                                          const DcpItem& it, const DcpCols& cols, Input& input,
-                                          Output& output, DcpGuard& guard) {
-  if constexpr (P < PD) {
-    dcp_iter<P, CHECK, ROWS>(ring, q, j, it, cols, input, output, guard);
-    dcp_iters<P + 1, CHECK, ROWS>(ring, q, j + 1, it, cols, input, output, guard);
-  }
-}
-
-// A single iteration of run-time phase r (alignment and tail), rows tested.
-template <int P, bool CHECK, class Input, class Output>
-__device__ __forceinline__ void dcp_iter_dyn(int r, T (&ring)[K > 1 ? K : 1][NR][C],
-                                             T (&q)[PD][C], int j, const DcpItem& it,
-                                             const DcpCols& cols,
-                                             Input& input, Output& output, DcpGuard& guard) {
-  if constexpr (P < PD) {
-    if (r == P) dcp_iter<P, CHECK, false>(ring, q, j, it, cols, input, output, guard);
-    else dcp_iter_dyn<P + 1, CHECK>(r, ring, q, j, it, cols, input, output, guard);
-  }
-}
-
-template <int P, bool CHECK, class Input>
-__device__ __forceinline__ void dcp_prefill(T (&q)[PD][C], int j0, const DcpItem& it,
-                                            const DcpCols& cols,
-                                            Input& input) {
-  if constexpr (P < PD) {
-    // the row in [j0, j0 + PD) that maps to slot P
-    dcp_fetch_row<CHECK, false>(q[P], j0 + dcp_mod(P - j0, PD), it, cols, input);
-    dcp_prefill<P + 1, CHECK>(q, j0, it, cols, input);
-  }
-}
-
-template <bool CHECK, class Input, class Output>
-__device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Input& input, Output& output,
+template <bool CHECK, class Pro, class Output>
+__device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Pro& pro, Output& output,
                                                 DcpGuard& guard, const T (&km)[DCP_NK]) {
+  extern __shared__ __align__(16) unsigned char dcp_smem[];
   const int lane = threadIdx.x & 31;
   DcpCols cols;
+  const int col0 = it.x0 - HX + lane * C;
+  cols.dst = (unsigned)__cvta_generic_to_shared(dcp_smem) +
+             (threadIdx.x >> 5) * (DCP_NIN * R * ROWB);
+  cols.ring = 0u;
 #pragma unroll
-  for (int k = 0; k < DCP_NK; ++k) cols.km[k] = km[k];
-  cols.col0 = it.x0 - K * DCP_RX + lane * C;
-#pragma unroll
-  for (int c = 0; c < C; ++c)
-    cols.keep[c] = (unsigned)(cols.col0 + c) < (unsigned)it.nx ? ~(typename DcpBits<T>::type)0 : 0;
-  T ring[K > 1 ? K : 1][NR][C];
-#pragma unroll
-  for (int l = 0; l < (K > 1 ? K : 1); ++l)
-#pragma unroll
-    for (int d = 0; d < NR; ++d)
-#pragma unroll
-      for (int c = 0; c < C; ++c) ring[l][d][c] = (T)0;
-  // Rows before the first streamed row hold zeros: exact ghosts above the
+  for (int c = 0; c < C; ++c) {
+    const int col = col0 + c;
+    if (CHECK) cols.ring |= col < DCP_RX || col >= it.nx - DCP_RX ? 1u << c : 0u;
+    cols.keep[c] = (unsigned)col < (unsigned)it.nx ? ~(typename DcpBits<T>::type)0 : 0;
+    if (CHECK && DCP_BC == DCP_BC_PERIODIC)
+      cols.pcol[c] = dcp_wrap(it.x0 - HX + lane + 32 * c, it.nx);
+  }
+  // Rows before the first streamed row count as zeros: exact ghosts above the
   // array; inside the array they only feed warm-up rows that are never written.
-  int j = it.y0 - K * DCP_RY;
-  const int jend = it.y1 + K * DCP_RY;
-  T q[PD][C];
-  dcp_prefill<0, CHECK>(q, j, it, cols, input);
-  // Iterations [jb0, jb1) touch only rows inside the array (and outside a
-  // fixed ring): level rows j - L*RY for L = 1..K, the fetched row j + PD and
-  // the written row j - K*RY in [y0, y1).  They run without row tests.
-  // One loop with one call site per form keeps the unrolled code small:
-  // PD-aligned groups inside [jb0, jb1) take the unchecked form, every other
-  // iteration (warm-up, alignment, tail) the row-checked one.
-  const int ring_w = DCP_BC == DCP_BC_FIXED_RING ? DCP_RY : 0;
-  const int jb0 = K * DCP_RY + max(it.y0, ring_w);
-  const int jb1 = min(min(it.y1 + K * DCP_RY, it.ny - ring_w + DCP_RY), it.ny - PD);
+  T st[K][NST][C];
+#pragma unroll
+  for (int l = 0; l < K; ++l)
+#pragma unroll
+    for (int d = 0; d < NST; ++d)
+#pragma unroll
+      for (int c = 0; c < C; ++c) st[l][d][c] = (T)0;
+  int j = it.y0 - K * RY;
+  const int jend = it.y1 + K * RY;
+  int slot = 0;
+  __syncwarp();  // the previous item's rows have been read
+  for (int r = 0; r < D; ++r) dcp_fetch_row<CHECK, false>(r, j + r, it, cols);
+  // Rows [f0, f1] run without row tests: every row such an iteration touches
+  // -- level rows from j - K*RY, the requested row j + D -- lies inside the
+  // array and outside a fixed ring (periodic: the requested row).
+  const int f0 = DCP_BC == DCP_BC_PERIODIC ? -D : K * RY + RING;
+  const int f1 = min(jend - 1, it.ny - (DCP_BC == DCP_BC_PERIODIC ? 0 : RING) - 1 - D);
   while (j < jend) {
-    if (j >= jb0 && j + PD <= jb1 && dcp_mod(j, PD) == 0) {
-      dcp_iters<0, CHECK, true>(ring, q, j, it, cols, input, output, guard);
-      j += PD;
-    } else {
-      dcp_iter_dyn<0, CHECK>(dcp_mod(j, PD), ring, q, j, it, cols, input, output, guard);
+    if (j >= f0) {
+#pragma unroll 1
+      for (; j < f1; j += 2) {  // pairs: the partial sums alternate registers
+        dcp_iter<CHECK, true>(st, slot, j, it, cols, km, pro, output, guard);
+        dcp_iter<CHECK, true>(st, slot, j + 1, it, cols, km, pro, output, guard);
+      }
+    }
+    if (j < jend) {
+      dcp_iter<CHECK, false>(st, slot, j, it, cols, km, pro, output, guard);
       ++j;
     }
   }
+  dcp_wait_copies<0>();
 }
 
 // Strips whose columns all lie inside the array (outside a fixed ring) take
 // the path without per-column boundary tests.
 // With DCP_GUARD every row the stream reads enters the magnitude guard.
-template <class Input, class Output>
-__device__ __forceinline__ void dcp_stream(const DcpItem& it, Input&& input, DcpGuard& guard,
+template <class Pro, class Output>
+__device__ __forceinline__ void dcp_stream(const DcpItem& it, Pro&& pro, DcpGuard& guard,
                                            const T (&km)[DCP_NK], Output&& output) {
   const int lo = DCP_BC == DCP_BC_FIXED_RING ? DCP_RX : 0;
-  const int first = it.x0 - K * DCP_RX;
-  if (first >= lo && first + SPAN <= it.nx - lo)
-    dcp_stream_impl<false>(it, input, output, guard, km);
-  else
-    dcp_stream_impl<true>(it, input, output, guard, km);
+  const int first = it.x0 - HX;
+  if (first >= lo && first + SPAN <= it.nx - lo) dcp_stream_impl<false>(it, pro, output, guard, km);
+  else dcp_stream_impl<true>(it, pro, output, guard, km);
 }
 
+// Bit c: the lane's column c is written by the strip starting at x0.
+__device__ __forceinline__ unsigned dcp_written(int x0, int nx) {
+  const int col0 = x0 - HX + (threadIdx.x & 31) * C;
+  unsigned m = 0u;
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const int col = col0 + c;
+    m |= col >= x0 && col < x0 + W && col < nx ? 1u << c : 0u;
+  }
+  return m;
+}
+
+__device__ __forceinline__ void dcp_write_row(T* p, const T (&v)[C], unsigned m, int run_vec) {
+  const int vec = DCP_VEC > 0 ? DCP_VEC : run_vec;
+  if (vec == C) dcp_st_row<C>(p, v, m);
+  else if (C > 2 && vec == 2) dcp_st_row<2>(p, v, m);
+  else dcp_st_row<1>(p, v, m);
+}
+
+#if !defined(DCP_PRO) || !defined(DCP_POST) || !defined(DCP_W)
+#error "incomplete generated prefix"
+#endif
+
 #if !DCP_BATCH
-// Single array: items = strips x row segments of p.seg rows.
+// Single array: items = strips x row segments of p.seg rows; the host launches
+// the variant whose DCP_VEC suits every buffer and the row length.
 extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(const DcpStParams p) {
   T sc[DCP_ARR(DCP_NSCALAR)];
 #pragma unroll
@@ -320,29 +373,39 @@ extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(co
   dcp_load_multipliers(km, dcp_km);
   for (int w = warp; w < items; w += nwarps) {
     const int sg = w / strips, st = w - sg * strips;
-    DcpItem it{nullptr, nullptr, ny, nx, st * W, sg * SEG, min(ny, (sg + 1) * SEG)};
-    const int col0 = it.x0 - K * DCP_RX + lane * C;
+    DcpItem it;
+#pragma unroll
+    for (int l = 0; l < DCP_NIN; ++l) it.in[l] = p.ld[l];
+    it.ny = ny;
+    it.nx = nx;
+    it.x0 = st * W;
+    it.y0 = sg * SEG;
+    it.y1 = min(ny, it.y0 + SEG);
+    it.vec = 0;
+    const int col0 = it.x0 - HX + lane * C;
+    const unsigned wm = dcp_written(it.x0, nx);
     dcp_stream(
-        it,
-        [&](long long gi) { return dcp_input(p, sc, gi); }, guard, km,
+        it, [&](const T (&ld)[DCP_NIN]) { return dcp_pro(ld, sc); }, guard, km,
         [&](int y, const T (&v)[C]) {
+          const long long gi = (long long)y * nx + col0;
+#if DCP_POST
+          T sv[DCP_ARR(DCP_NSTORE)][C];
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            const int col = col0 + c;
-            if (col < it.x0 || col >= it.x0 + W || col >= nx) continue;
-            const long long gi = (long long)y * nx + col;
-#if DCP_LAST
+            if (!((wm >> c) & 1u)) continue;
             T stv[DCP_ARR(DCP_NSTORE)], rv[DCP_ARR(DCP_NRED)];
-            dcp_post(p, sc, gi, v[c], stv, rv);
+            dcp_post(p, sc, gi + c, v[c], stv, rv);
 #pragma unroll
-            for (int s = 0; s < DCP_NSTORE; ++s) p.st[s][gi] = stv[s];
+            for (int s = 0; s < DCP_NSTORE; ++s) sv[s][c] = stv[s];
 #pragma unroll
             for (int r = 0; r < DCP_NRED; ++r)
               acc[r] = dcp_red_comb(dcp_red_op(r), acc[r], dcp_red_lift(dcp_red_op(r), rv[r]));
-#else
-            p.st[0][gi] = v[c];
-#endif
           }
+#pragma unroll
+          for (int s = 0; s < DCP_NSTORE; ++s) dcp_write_row(p.st[s] + gi, sv[s], wm, 0);
+#else
+          dcp_write_row(p.st[0] + gi, v, wm, 0);
+#endif
         });
   }
 #if DCP_LAST && DCP_NRED > 0
@@ -387,21 +450,24 @@ extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(co
     const DcpInst I = p.inst[lo];
     const int t = w - I.tile0;
     const int sg = t / I.tiles_x, st = t - sg * I.tiles_x;
-    DcpItem it{I.in, I.out, I.ny, I.nx, st * W, sg * p.seg, min(I.ny, (sg + 1) * p.seg)};
-    const T* in = I.in;
-    T* out = I.out;
-    const int col0 = it.x0 - K * DCP_RX + lane * C;
+    DcpItem it;
+    it.in[0] = I.in;
+    it.ny = I.ny;
+    it.nx = I.nx;
+    it.x0 = st * W;
+    it.y0 = sg * p.seg;
+    it.y1 = min(I.ny, it.y0 + p.seg);
+    // the widest access that suits both buffers and the row length
+    const unsigned long long mis = reinterpret_cast<unsigned long long>(I.in) |
+                                   reinterpret_cast<unsigned long long>(I.out) |
+                                   (unsigned long long)I.nx * sizeof(T);
+    it.vec = (mis & 15) == 0 ? C : (C > 2 && (mis & 7) == 0 ? 2 : 1);
+    T* out = I.out + it.x0 - HX + lane * C;
+    const int nx = I.nx, vec = it.vec;
+    const unsigned wm = dcp_written(it.x0, nx);
     dcp_stream(
-        it,
-        [&](long long gi) { return in[gi]; }, guard, km,
-        [&](int y, const T (&v)[C]) {
-#pragma unroll
-          for (int c = 0; c < C; ++c) {
-            const int col = col0 + c;
-            if (col < it.x0 || col >= it.x0 + W || col >= it.nx) continue;
-            out[(long long)y * it.nx + col] = v[c];
-          }
-        });
+        it, [&](const T (&ld)[DCP_NIN]) { return ld[0]; }, guard, km,
+        [&](int y, const T (&v)[C]) { dcp_write_row(out + (long long)y * nx, v, wm, vec); });
   }
 #if DCP_GUARD
   guard.flush(p.guard);

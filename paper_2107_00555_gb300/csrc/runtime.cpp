@@ -261,16 +261,21 @@ static void* dalloc(GraphImpl::Runtime& rt, size_t bytes) {
   return p;
 }
 
-static void load_launch(LaunchSpec& ls) {
-  ls.fn = load_function(ls.code.source, ls.code.name, nullptr, &ls.regs);
-  if (ls.code.smem_bytes > 48 * 1024)
-    check_cu(drv().funcSetAttribute(ls.fn, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES,
-                                    ls.code.smem_bytes),
+// Allows a kernel its dynamic shared memory; CTAs resident per SM.
+static int prepare_function(CUfunction fn, const CodegenOut& code) {
+  if (code.smem_bytes > 48 * 1024)
+    check_cu(drv().funcSetAttribute(fn, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES,
+                                    code.smem_bytes),
              "cuFuncSetAttribute(max dynamic smem)");
   int occ = 0;
-  check_cu(drv().occupancy(&occ, ls.fn, ls.code.threads, ls.code.smem_bytes), "occupancy query");
-  if (occ < 1) fail(DCP_E_UNSUPPORTED, "kernel " + ls.code.name + " cannot be resident on an SM");
-  ls.occupancy = occ;
+  check_cu(drv().occupancy(&occ, fn, code.threads, code.smem_bytes), "occupancy query");
+  if (occ < 1) fail(DCP_E_UNSUPPORTED, "kernel " + code.name + " cannot be resident on an SM");
+  return occ;
+}
+
+static void load_launch(LaunchSpec& ls) {
+  ls.fn = load_function(ls.code.source, ls.code.name, nullptr, &ls.regs);
+  ls.occupancy = prepare_function(ls.fn, ls.code);
 }
 
 static void ensure_device(GraphImpl& g) {
@@ -566,13 +571,28 @@ static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const
   }
   for (size_t i = 0; i < G.scalars.size(); ++i) p.sc[i] = ptr[G.scalars[i]];
   const int nd = (int)G.shape.size();
+  CUfunction fn = ls.fn;
+  int occ = ls.occupancy;
   int64_t gx;
   if (G.variant == 1) {
     // warp stream: one warp per (strip, row segment) work item, warps stride
-    const int W = stream_width(G);
+    // the kernel's access width suits the row length; buffers off its boundary
+    // take the element-wise variant
+    uintptr_t mis = 0;
+    for (int i = 0; i < kMaxIO; ++i) mis |= (uintptr_t)p.ld[i] | (uintptr_t)p.st[i];
+    if (mis % (uintptr_t)(ls.code.vec * dtype_size(G.dtype))) {
+      if (!ls.fn_scalar) {
+        ls.code_scalar = gen_stencil_kernel(g, G, ls.s0, ls.s1, 1);
+        ls.fn_scalar = load_function(ls.code_scalar.source, ls.code_scalar.name, nullptr, nullptr);
+        ls.occ_scalar = prepare_function(ls.fn_scalar, ls.code_scalar);
+      }
+      fn = ls.fn_scalar;
+      occ = ls.occ_scalar;
+    }
+    const int W = stream_width(G, ls.s1 - ls.s0);
     int64_t items = (int64_t)((p.nx + W - 1) / W) * ((p.ny + G.seg - 1) / G.seg);
     const int wpb = ls.code.threads / 32;
-    int64_t warps = std::min<int64_t>(items, (int64_t)rt.sms * ls.occupancy * wpb);
+    int64_t warps = std::min<int64_t>(items, (int64_t)rt.sms * occ * wpb);
     gx = std::max<int64_t>(1, (warps + wpb - 1) / wpb);
     p.tiles_x = p.tiles_y = p.tiles_z = 1;
     p.seg = G.seg;
@@ -594,7 +614,7 @@ static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const
     return;
   }
   void* args[] = {&p};
-  check_cu(drv().launchKernel(ls.fn, (unsigned)gx, (unsigned)p.tiles_z, 1, ls.code.threads, 1, 1,
+  check_cu(drv().launchKernel(fn, (unsigned)gx, (unsigned)p.tiles_z, 1, ls.code.threads, 1, 1,
                               ls.code.smem_bytes, (CUstream)s, args, nullptr),
            "cuLaunchKernel(stencil)");
 }
@@ -671,11 +691,11 @@ static void launch_batch(GraphImpl& g, LaunchSpec& ls, const std::vector<const v
     void* out_slab = last ? nullptr : group_state(g, ls.group, chunk % 2);
     // members ordered by tile count, largest first, for load balance
     // work items of a member: tiles (tile kernel) or column strips (stream kernel)
+    const int W = stream_width(G, ls.s1 - ls.s0);
     auto tiles_of = [&](int k) {
       const Group& M = g.batch_store[G.batch_members[k]];
       int64_t ny = M.shape[0], nx = M.shape[1];
-      if (G.variant == 1)
-        return ((nx + stream_width(G) - 1) / stream_width(G)) * ((ny + G.seg - 1) / G.seg);
+      if (G.variant == 1) return ((nx + W - 1) / W) * ((ny + G.seg - 1) / G.seg);
       return ((nx + G.tile[2] - 1) / G.tile[2]) * ((ny + G.tile[1] - 1) / G.tile[1]);
     };
     std::vector<int> order(nm);
@@ -692,7 +712,7 @@ static void launch_batch(GraphImpl& g, LaunchSpec& ls, const std::vector<const v
       I.out = last ? const_cast<void*>(ptr[M.st_out]) : (char*)out_slab + off;
       I.ny = (int32_t)M.shape[0];
       I.nx = (int32_t)M.shape[1];
-      I.tiles_x = (int32_t)(G.variant == 1 ? (I.nx + stream_width(G) - 1) / stream_width(G)
+      I.tiles_x = (int32_t)(G.variant == 1 ? (I.nx + W - 1) / W
                                            : (I.nx + G.tile[2] - 1) / G.tile[2]);
       I.tile0 = (int32_t)t0;
       t0 += tiles_of(k);
@@ -941,7 +961,7 @@ void apply_config(GraphImpl& g, int gi, const TuneCfg& cfg) {
       G.seg = cfg[2] > 0 ? cfg[2] : 64;
     } else {
       int64_t ny = G.shape.size() == 2 ? G.shape[0] : 1, nx = G.shape.back();
-      int64_t strips = (nx + stream_width(G) - 1) / stream_width(G);
+      int64_t strips = (nx + stream_width(G, G.depth) - 1) / stream_width(G, G.depth);
       int64_t seg = cfg[2] > 0 ? cfg[2]
                                : std::max<int64_t>((ny * strips + 2431) / 2432,
                                                    8 * G.depth * std::max(1, G.radius[1]));
