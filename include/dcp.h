@@ -122,13 +122,13 @@ enum {
   DCP_OPT_STREAM_ROWS = 9,     /* warp-stream stencils: rows per work item (>= 1) */
   DCP_OPT_TILE_Z = 10,         /* 3-D stencils: planes per CTA (z chunk, 1..1024) */
   DCP_OPT_STREAM_PREFETCH = 11, /* warp-stream stencils: row windows requested ahead (1..4) */
-  DCP_OPT_STREAM_THREADS = 12, /* warp-stream stencils: threads per CTA (32..1024, multiple of 32; default 64) */
+  DCP_OPT_STREAM_THREADS = 12, /* warp-stream stencils: threads per CTA (32..1024, multiple of 32; default 32) */
   DCP_OPT_CELLS_PER_THREAD = 13, /* 3-D stencils: cells per thread along x (1 or 2) */
   DCP_OPT_MAP_UNROLL = 14,      /* map kernels: 16-byte vectors per array in flight per thread (1..8) */
   DCP_OPT_DEFERRED_WEIGHT = 15, /* stencils: 1 (default) deferred common weight where it applies,
                                    0 the plain weighted sum everywhere (set before dcp_fuse) */
   DCP_OPT_STREAM_MIN_CTAS = 16, /* warp-stream stencils: CTAs per SM the register budget must
-                                   allow (1..32; default: the compiler's choice) */
+                                   allow (1..32; default: four warps per scheduler where the plan counts on them) */
   DCP_OPT_ADJOINT_DEPTH = 17    /* reverse pass of 1-D / 2-D stencil chains with step
                                    epilogues: k >= 1 runs k reverse steps per launch from every
                                    k-th state, recomputing the forward states in the tile; 0

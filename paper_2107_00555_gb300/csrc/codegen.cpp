@@ -810,7 +810,8 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
   // 512 bytes each; fewer rows, then fewer warps per CTA where 192 KB is short
   const int nload = pro ? (int)G.loads.size() : 1;
   const int nin = std::max(1, nload);  // a prologue of broadcast scalars loads no array
-  int threads = G.threads, ring = 8 * G.prefetch;
+  int threads = G.threads, ring = 8;  // a power of two
+  while (ring < 8 * G.prefetch) ring *= 2;
   auto smem = [&] { return threads / 32 * nin * ring * 512; };
   while (smem() > 192 * 1024 && ring > 4) ring /= 2;
   while (smem() > 192 * 1024 && threads > 32) threads = threads / 64 * 32;

@@ -515,13 +515,197 @@ struct Planner {
     return it == g.options.end() ? def : it->second;
   }
 
+  // Issue cycles of one operation on the C columns a lane holds (binary64
+  // operations cost the FP64 pipe 64 cycles per warp and scheduler).
+  double op_cycles(int op, int dtype) const {
+    if (dtype == DCP_F64) {
+      const double n = op == DCP_EXP || op == DCP_SQRT || op == DCP_DIV ? 10
+                       : op == DCP_SIN || op == DCP_COS                ? 15
+                       : op == DCP_TANH                                ? 7 : 1;
+      return 2 * 64 * n;
+    }
+    const double n = op == DCP_EXP || op == DCP_SQRT || op == DCP_DIV ? 10
+                     : op == DCP_SIN || op == DCP_COS || op == DCP_TANH ? 25 : 1;
+    return 4 * n;
+  }
+
+  // Cycles of one launch of K steps of the warp-stream kernel, and the rows
+  // per work item that give them: nw warps per scheduler (4 per SM) stream
+  // seg + 2 K ry rows each, a row taking the larger of its latency and the
+  // nw warps' issue.  Fitted to 24 steps on 64^2 .. 4000 x 4100 binary32 and
+  // 64^2 .. 2047 x 2051 binary64 grids (within 15 %): binary32 issues 27
+  // cycles per level and 42 per row with a latency of 45 per level and 130
+  // per row; binary64 is bound by the FP64 pipe (p operations on 2 columns),
+  // with a latency of 500 per level and 300 per row.
+  double stream_cycles(const Group& G, int K, int64_t& seg, int& nw) const {
+    const int64_t ny = G.shape.size() == 2 ? G.shape[0] : 1, nx = G.shape.back();
+    const int ry = G.shape.size() == 2 ? G.radius[1] : 0;
+    const int W = stream_width(G, K);
+    const int64_t strips = (nx + W - 1) / W;
+    const int pts = (int)G.offsets.size() / 3;
+    double issue, latency;
+    if (G.dtype == DCP_F64) {
+      issue = K * 2.0 * 64 * std::max(2, pts - 1) + 60;
+      latency = 300.0 + 500.0 * K;
+    } else {
+      issue = K * (7.0 + 4.0 * pts) + 42;
+      latency = 130.0 + 45.0 * K;
+    }
+    double epi = 0;
+    for (const StepDesc& st : G.steps)
+      for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
+    issue += K * epi / (double)G.steps.size();
+    for (int m : G.members) issue += op_cycles(g.nodes[m].op, G.dtype);
+    const int64_t cells = ny * nx;
+    const double bytes = 2.0 * cells * dtype_size(G.dtype);
+    // 3237 bytes per clock from HBM (6.7 TB/s at 2.07 GHz), about twice that
+    // where both arrays stay in L2
+    const double mem = bytes / (bytes > 100e6 ? 3237.0 : 6500.0);
+    double best = 1e300;
+    const int64_t slots = 152 * 4;
+    for (int n = 1; n <= 4; ++n) {
+      const int64_t segs = std::max<int64_t>(1, std::min<int64_t>(ny, n * slots / strips));
+      const int64_t sg = (ny + segs - 1) / segs;
+      const int64_t items = strips * ((ny + sg - 1) / sg);
+      const int64_t per = (items + slots - 1) / slots;  // warps one scheduler runs
+      const int64_t waves = (per + n - 1) / n;
+      const double c = std::max(mem, (double)waves * (sg + 2 * K * ry) * std::max(latency, issue * std::min<int64_t>(per, n)));
+      if (c < best * 0.999) best = c, seg = sg, nw = n;
+    }
+    return best;
+  }
+
+  // Cycles of one batched launch of K steps with seg rows per work item: the
+  // issue of every item's rows over the 608 schedulers plus half an item's
+  // time for the uneven end, at least one item's latency.  (4096 binary32
+  // instances of 32^2 to 512^2, 20 steps at 5 per launch: 32, 64, 128 and 256
+  // rows took 2.51, 2.23, 2.18 and 2.24 ms.)
+  double batch_cycles(const Group& G, int K, int seg) const {
+    const int W = stream_width(G, K), ry = G.radius[1];
+    const int pts = (int)G.offsets.size() / 3;
+    const bool f64 = G.dtype == DCP_F64;
+    double epi = 0;
+    for (const StepDesc& st : G.steps)
+      for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
+    const double issue = (f64 ? K * 2.0 * 64 * std::max(2, pts - 1) + 60 : K * (11.0 + 4.0 * pts) + 100) +
+                         K * epi / (double)G.steps.size();
+    const double latency = f64 ? 300.0 + 500.0 * K : 130.0 + 45.0 * K;
+    double rows = 0, bytes = 0;
+    int64_t items = 0, longest = 1;
+    for (int m : G.batch_members) {
+      const Group& M = batch_store[m];
+      const int64_t ny = M.shape[0], nx = M.shape[1];
+      if (ny * nx == 0) continue;
+      const int64_t strips = (nx + W - 1) / W, segs = (ny + seg - 1) / seg;
+      rows += (double)strips * (ny + segs * 2 * K * ry);
+      items += strips * segs;
+      longest = std::max(longest, std::min<int64_t>(ny, seg) + 2 * K * ry);
+      bytes += 2.0 * ny * nx * dtype_size(G.dtype);
+    }
+    const double n = std::min(4.0, items / 608.0);
+    const double c = std::max(rows * issue / 608 + 0.5 * longest * std::max(latency, n * issue),
+                              longest * latency);
+    return std::max(c, bytes / (bytes > 100e6 ? 3237.0 : 6500.0));
+  }
+
+  // Cycles of one launch of K steps of the shared-memory tile kernel (256
+  // threads per CTA), fitted to the same runs: a step takes about 290 cycles
+  // per 256 cells of its region (binary32, two CTAs per SM in parallel) or, on
+  // binary64, 1200 plus the region's operations at 2 per clock.
+  double tile_cycles(const Group& G, int K, int ty, int tx) const {
+    const int64_t ny = G.shape[0], nx = G.shape[1];
+    const int64_t tiles = ((ny + ty - 1) / ty) * ((nx + tx - 1) / tx);
+    const int64_t per = (tiles + 151) / 152;  // tiles of one SM
+    const int pts = (int)G.offsets.size() / 3;
+    double t = 0, epi = 0;
+    for (const StepDesc& st : G.steps)
+      for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
+    epi /= (double)G.steps.size();
+    for (int s = 0; s < K; ++s) {
+      const double cells = (double)(ty + 2 * (K - 1 - s) * G.radius[1]) * (tx + 2 * (K - 1 - s) * G.radius[2]);
+      if (G.dtype == DCP_F64) t += 1200 + per * cells * (std::max(1, pts - 1) + epi / 128) / 2;
+      else t += std::max(1.0, per / 2.0) * (290.0 * pts / 5 + 0.6 * epi) * std::ceil(cells / 256);
+    }
+    return t;
+  }
+
+  // Kernel form, depth, rows per work item or tile of a 1-D / 2-D stencil
+  // group, each unless an option sets it.
   void choose_stencil_tiling(Group& G) {
     choose_stencil_tiling_impl(G);
+    const int nd = G.kind == GroupKind::Batch ? 2 : (int)G.shape.size();
+    if (nd == 3) {
+      G.variant = 0;
+      return;
+    }
+    const auto has = [&](int key) { return g.options.count(key) > 0; };
+    const int S = (int)G.steps.size();
+    const bool tt = (flags & DCP_TIME_TILE) != 0;
+    const bool free_depth = tt && !has(DCP_OPT_TIME_TILE_DEPTH);
+    // launches of equal depth: at most `most` steps each
+    auto even = [S](int most) {
+      const int n = (S + most - 1) / most;
+      return (S + n - 1) / n;
+    };
+    // a launch costs about 3 us (6200 cycles) besides its rows
+    const double launch = 6200;
+    const int64_t cells = G.kind == GroupKind::Batch ? 0 : G.shape.size() == 2 ? G.shape[0] * G.shape[1] : G.shape[0];
     // the warp-stream kernel when it applies (1-D or 2-D, radius <= 2); the
     // shared-memory tile kernel otherwise
     int var = stream_eligible(G, G.depth) ? 1 : 0;
     auto it = g.options.find(DCP_OPT_STENCIL_KERNEL);
     if (it != g.options.end()) var = (it->second == 1 && stream_eligible(G, G.depth)) ? 1 : 0;
+    int64_t seg = 0;
+    int nw = 4;
+    if (G.kind == GroupKind::Stencil && var == 1 && cells > 0) {
+      double best = stream_cycles(G, G.depth, seg, nw) + launch;
+      best *= (S + G.depth - 1) / G.depth;
+      if (free_depth)
+        for (int most = 1; most <= std::min(S, G.dtype == DCP_F32 ? 10 : 4); ++most) {
+          const int K = even(most);
+          int64_t sg;
+          int n;
+          if (!stream_eligible(G, K)) continue;
+          const double c = (stream_cycles(G, K, sg, n) + launch) * ((S + K - 1) / K);
+          if (c < best) best = c, G.depth = K, seg = sg, nw = n;
+        }
+      // Small grids run faster in shared-memory tiles, where every cell of a
+      // step is in flight at once (256^2 binary64, 24 steps: 46 us against 91;
+      // 64^2 binary32: 17 against 25); from 512^2 on the stream wins.
+      if (nd == 2 && cells <= 512 * 512 && !has(DCP_OPT_STENCIL_KERNEL) && !has(DCP_OPT_TILE_X) &&
+          !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS)) {
+        for (int most = 1; most <= std::min(S, 12); ++most) {
+          const int K = free_depth ? even(most) : G.depth;
+          for (int tx : {16, 32})
+            for (int ty : {4, 8, 12, 14, 16, 24, 32}) {
+              const long smem = 2L * (ty + 2 * K * G.radius[1]) * (tx + 2 * K * G.radius[2]) * dtype_size(G.dtype);
+              if (smem > 96 * 1024) continue;
+              const double c = (tile_cycles(G, K, ty, tx) + 1.3 * launch) * ((S + K - 1) / K);
+              if (c < best) {
+                best = c;
+                var = 0;
+                G.depth = K;
+                G.tile[1] = ty;
+                G.tile[2] = tx;
+              }
+            }
+          if (!free_depth) break;
+        }
+      }
+    }
+    if (G.kind == GroupKind::Batch && var == 1) {
+      double best = 1e300;
+      const int most0 = free_depth ? 1 : G.depth;
+      const int most1 = free_depth ? std::min(S, G.dtype == DCP_F32 ? 8 : 3) : G.depth;
+      for (int most = most0; most <= most1; ++most) {
+        const int K = free_depth ? even(most) : G.depth;
+        if (!stream_eligible(G, K)) continue;
+        for (int sg : {16, 32, 64, 128, 256}) {
+          const double c = (batch_cycles(G, K, sg) + launch) * ((S + K - 1) / K);
+          if (c < best) best = c, G.depth = K, seg = sg;
+        }
+      }
+    }
     if (it != g.options.end() && it->second == 2 && G.kind == GroupKind::Stencil &&
         G.shape.size() <= 2) {
       // cooperative form: every step in one launch on the tile the options
@@ -538,22 +722,13 @@ struct Planner {
     }
     G.variant = var;
     if (var == 1) {
-      G.threads = (int)opt(DCP_OPT_STREAM_THREADS, 64);
+      // one warp per CTA: work items end at different times, and a CTA's
+      // slots free together (batch of 4096 instances 2.28 -> 2.13 ms)
+      G.threads = (int)opt(DCP_OPT_STREAM_THREADS, 32);
       G.prefetch = (int)opt(DCP_OPT_STREAM_PREFETCH, 1);
-      G.min_ctas = (int)opt(DCP_OPT_STREAM_MIN_CTAS, 0);
-      if (G.kind == GroupKind::Batch) {
-        G.seg = 64;  // rows per work item: short, uniform items balance the batch
-      } else {
-        // rows per work item: enough items to fill the GPU, and at least
-        // 8 * depth * radius rows so warm-up rows stay a small fraction
-        int64_t ny = G.shape.size() == 2 ? G.shape[0] : 1;
-        int64_t nx = G.shape.back();
-        int64_t strips = (nx + stream_width(G, G.depth) - 1) / stream_width(G, G.depth);
-        int64_t target_items = 152 * 16;
-        int64_t seg = (ny * strips + target_items - 1) / target_items;
-        seg = std::max<int64_t>(seg, 8 * G.depth * std::max(1, G.radius[1]));
-        G.seg = (int)std::min<int64_t>(std::max<int64_t>(seg, 1), std::max<int64_t>(ny, 1));
-      }
+      // registers for the four warps per scheduler the plan counts on
+      G.min_ctas = (int)opt(DCP_OPT_STREAM_MIN_CTAS, nw >= 4 ? std::min(32, 512 / G.threads) : 0);
+      G.seg = (int)std::max<int64_t>(seg, 1);
       auto so = g.options.find(DCP_OPT_STREAM_ROWS);
       if (so != g.options.end()) G.seg = (int)so->second;
     }

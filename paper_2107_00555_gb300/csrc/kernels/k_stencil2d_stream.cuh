@@ -18,10 +18,11 @@
 // scoreboards, and the lane exchanges need them too.)
 //
 // Measured on a GB300 against the form that kept 2*RY + 1 rows per level and
-// read them element by element: 4000 x 4100 binary32, fixed ring, 50 steps, 4
-// per launch 526 -> 369 us; 2047 x 2051 binary64, periodic, 20 steps, 2 per
-// launch 722 (shared-memory tiles) -> 594 us; the 20-step reverse pass of a
-// 4096^2 binary32 chain with its loss, one step per launch, 3.01 -> 1.79 ms.
+// read them element by element (with the planner's depth and rows per item):
+// 4000 x 4100 binary32, fixed ring, 50 steps 526 -> 295 us; 2047 x 2051
+// binary64, periodic, 20 steps 721 (shared-memory tiles) -> 572 us; 4096
+// binary32 instances of 32^2 to 512^2, 20 steps 2.84 -> 2.01 ms; the 20-step
+// reverse pass of a 4096^2 binary32 chain with its loss 3.01 -> 1.71 ms.
 //
 // Work items are (array, strip, row segment); a segment streams its rows plus
 // NSTEPS*RY warm-up rows above and below it.  Warps stride through the items
@@ -88,11 +89,11 @@ template <> struct DcpAcc<1> { typedef T type; };
 template <> struct DcpAcc<2> { typedef typename DcpVec2<T>::type type; };
 template <> struct DcpAcc<4> { typedef uint4 type; };  // C = 4: binary32
 
-// Asynchronous copy of V elements into the ring (zeros when !ok).
+// Asynchronous copy of V elements into the ring: `n` bytes of them from src
+// (all or none), zeros for the rest.
 template <int V>
-__device__ __forceinline__ void dcp_copy(unsigned dst, const T* src, bool ok) {
+__device__ __forceinline__ void dcp_copy(unsigned dst, const T* src, int n) {
   constexpr int B = V * (int)sizeof(T);
-  const int n = ok ? B : 0;
   if constexpr (B == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
   else
@@ -117,10 +118,11 @@ struct DcpCols {
   int col0;
   unsigned ring;                       // bit c: the column belongs to a fixed ring
   typename DcpBits<T>::type keep[C];   // all ones inside the array, else 0
-  // copies: access i of the lane covers columns lane + 32 i of the strip in
-  // units of V elements, so that a warp's copies are contiguous
+  // Copies: access i of a lane covers unit lane + 32 i of the strip (units of V
+  // elements), so that a warp's copies are contiguous.
+  unsigned in;                         // bit i: access i lies inside the array
   int pcol[C];                         // periodic CHECK strips: the wrapped column of access i (V = 1)
-  unsigned dst;                        // shared address of the warp's ring
+  unsigned dst;                        // shared address of the warp's ring, at the lane's vector
 };
 
 // CHECK: the strip reaches outside the array (per-column tests).  ROWS: every
@@ -173,73 +175,93 @@ __device__ __forceinline__ void dcp_st_row(T* p, const T (&src)[C], unsigned in)
   }
 }
 
-// Requests a row (V elements per copy) from p, the strip's first column.
+// Copies of one row: p points at the lane's first unit, dst at the lane's
+// 16-byte vector of the ring row.
 template <int V, bool CHECK>
-__device__ __forceinline__ void dcp_fetch_units(unsigned dst, const T* row, int first, int nx,
-                                                bool row_ok) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void dcp_copy_row(unsigned dst, const T* p, unsigned in) {
+  constexpr int B = V * (int)sizeof(T);
+  dst -= (threadIdx.x & 31) * (16 - B);
 #pragma unroll
-  for (int i = 0; i < C / V; ++i) {
-    const int e = (lane + 32 * i) * V;
-    const bool ok = row_ok && (!CHECK || (unsigned)(first + e) < (unsigned)nx);
-    dcp_copy<V>(dst + e * (int)sizeof(T), ok ? row + first + e : row, ok);
-  }
+  for (int i = 0; i < C / V; ++i)
+    dcp_copy<V>(dst + 32 * i * B, p + 32 * i * V, !CHECK || ((in >> i) & 1u) ? B : 0);
 }
 
-// Requests input row j into ring slot `slot` (zeros outside the array).
-template <bool CHECK, bool ROWS>
-__device__ __forceinline__ void dcp_fetch_row(int slot, int j, const DcpItem& it,
-                                              const DcpCols& cols) {
-  const bool row_ok = ROWS || DCP_BC == DCP_BC_PERIODIC || (unsigned)j < (unsigned)it.ny;
-  const int row = ROWS ? j : (DCP_BC == DCP_BC_PERIODIC ? dcp_wrap(j, it.ny) : (row_ok ? j : 0));
-  const int first = it.x0 - HX;
+// Elements per copy of the strip.
+template <bool CHECK>
+__device__ __forceinline__ int dcp_vec(const DcpItem& it) {
+  if (DCP_BC == DCP_BC_PERIODIC && CHECK) return 1;
+  return DCP_VEC > 0 ? DCP_VEC : it.vec;
+}
+
+// Requests row `row` of the array (src: its first unit of the lane, per input)
+// into ring row `so`; CHECK: only the accesses of `in`.
+template <bool CHECK>
+__device__ __forceinline__ void dcp_request(unsigned so, const T* const (&src)[DCP_NIN], unsigned in,
+                                            const DcpItem& it, const DcpCols& cols) {
 #pragma unroll
   for (int l = 0; l < DCP_NLOAD; ++l) {
-    const T* p = it.in[l] + (long long)row * it.nx;
-    const unsigned dst = cols.dst + (l * R + slot) * ROWB;
-    const int vec = DCP_VEC > 0 ? DCP_VEC : it.vec;
+    const unsigned dst = cols.dst + l * (R * ROWB) + so;
     if (DCP_BC == DCP_BC_PERIODIC && CHECK) {
+      // src: the row's first column
 #pragma unroll
       for (int i = 0; i < C; ++i)
-        dcp_copy<1>(dst + ((threadIdx.x & 31) + 32 * i) * (int)sizeof(T), p + cols.pcol[i], true);
-    } else if (vec == C) {
-      dcp_fetch_units<C, CHECK>(dst, p, first, it.nx, row_ok);
-    } else if (C > 2 && vec == 2) {
-      dcp_fetch_units<2, CHECK>(dst, p, first, it.nx, row_ok);
+        dcp_copy<1>(dst - (threadIdx.x & 31) * (16 - (int)sizeof(T)) + 32 * i * (int)sizeof(T),
+                    src[l] + cols.pcol[i], (int)sizeof(T));
     } else {
-      dcp_fetch_units<1, CHECK>(dst, p, first, it.nx, row_ok);
+      const int vec = dcp_vec<CHECK>(it);
+      if (vec == C) dcp_copy_row<C, CHECK>(dst, src[l], in);
+      else if (C > 2 && vec == 2) dcp_copy_row<2, CHECK>(dst, src[l], in);
+      else dcp_copy_row<1, CHECK>(dst, src[l], in);
     }
   }
   dcp_commit();
 }
 
-__device__ __forceinline__ int dcp_next_slot(int s) { return s + 1 == R ? 0 : s + 1; }
+// The lane's first unit of row `row` in every input (periodic CHECK strips:
+// the row's first column).
+template <bool CHECK>
+__device__ __forceinline__ void dcp_src(const T* (&src)[DCP_NIN], int row, const DcpItem& it) {
+  const long long at = (long long)row * it.nx +
+                       (DCP_BC == DCP_BC_PERIODIC && CHECK
+                            ? 0 : it.x0 - HX + (int)(threadIdx.x & 31) * dcp_vec<CHECK>(it));
+#pragma unroll
+  for (int l = 0; l < DCP_NLOAD; ++l) src[l] = it.in[l] + at;
+}
 
-// One stream iteration: input row j from ring slot `slot`; row j + D is
-// requested into the slot that row j - 1 has left.
-template <bool CHECK, bool ROWS, class Pro, class Output>
-__device__ __forceinline__ void dcp_iter(T (&st)[K][NST][C], int& slot, int j, const DcpItem& it,
-                                         const DcpCols& cols, const T (&km)[DCP_NK], Pro& pro,
-                                         Output& output, DcpGuard& guard) {
-  dcp_wait_copies<D - 1>();  // this lane's copies of row j have landed
-  __syncwarp();              // every lane's have, and row j - 1 has been read
-  T a[C];
-  {
-    union { uint4 v; T t[C]; } x[DCP_NIN];
-    if (DCP_NLOAD == 0) x[0].v = make_uint4(0u, 0u, 0u, 0u);
+// Requests input row j with its boundary tests (zeros outside the array).
+template <bool CHECK>
+__device__ __forceinline__ void dcp_request_checked(unsigned so, int j, const DcpItem& it,
+                                                    const DcpCols& cols) {
+  const bool inside = (unsigned)j < (unsigned)it.ny;
+  const T* src[DCP_NIN];
+  dcp_src<CHECK>(src, DCP_BC == DCP_BC_PERIODIC ? dcp_wrap(j, it.ny) : (inside ? j : 0), it);
+  if (DCP_BC == DCP_BC_PERIODIC) dcp_request<CHECK>(so, src, cols.in, it, cols);
+  else dcp_request<true>(so, src, inside ? cols.in : 0u, it, cols);
+}
+
+constexpr unsigned RMASK = R * ROWB - 1;  // ring offsets wrap by a mask
+static_assert((R & (R - 1)) == 0, "power-of-two ring");
+
+// Input row j from ring row `so` through every level; `a` ends as row
+// j - K*RY after the last.
+template <bool CHECK, bool ROWS, class Pro>
+__device__ __forceinline__ void dcp_row(T (&a)[C], T (&st)[K][NST][C], unsigned so, int j,
+                                        const DcpItem& it, const DcpCols& cols,
+                                        const T (&km)[DCP_NK], Pro& pro, DcpGuard& guard) {
+  union { uint4 v; T t[C]; } x[DCP_NIN];
+  if (DCP_NLOAD == 0) x[0].v = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-    for (int l = 0; l < DCP_NLOAD; ++l)
-      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                   : "=r"(x[l].v.x), "=r"(x[l].v.y), "=r"(x[l].v.z), "=r"(x[l].v.w)
-                   : "r"(cols.dst + (l * R + slot) * ROWB + (threadIdx.x & 31) * 16)
-                   : "memory");
+  for (int l = 0; l < DCP_NLOAD; ++l)
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(x[l].v.x), "=r"(x[l].v.y), "=r"(x[l].v.z), "=r"(x[l].v.w)
+                 : "r"(cols.dst + l * (R * ROWB) + so)
+                 : "memory");
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      T ld[DCP_NIN];
+  for (int c = 0; c < C; ++c) {
+    T ld[DCP_NIN];
 #pragma unroll
-      for (int l = 0; l < DCP_NIN; ++l) ld[l] = x[l].t[c];
-      a[c] = pro(ld);
-    }
+    for (int l = 0; l < DCP_NIN; ++l) ld[l] = x[l].t[c];
+    a[c] = pro(ld);
   }
   if (DCP_PRO && DCP_BC != DCP_BC_PERIODIC) {
     // the maps of the zeros read outside the array need not be 0
@@ -255,11 +277,7 @@ __device__ __forceinline__ void dcp_iter(T (&st)[K][NST][C], int& slot, int j, c
 #pragma unroll
     for (int c = 0; c < C; ++c) guard.see(a[c]);
   }
-  dcp_fetch_row<CHECK, ROWS>(slot == 0 ? R - 1 : slot - 1, j + D, it, cols);
-  slot = dcp_next_slot(slot);
   dcp_levels<0, CHECK, ROWS>(a, st, j, it, cols, km);
-  const int y = j - K * RY;
-  if (y >= it.y0 && y < it.y1) output(y, a);
 }
 
 template <bool CHECK, class Pro, class Output>
@@ -270,15 +288,17 @@ __device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Pro& pro, Out
   DcpCols cols;
   const int col0 = it.x0 - HX + lane * C;
   cols.dst = (unsigned)__cvta_generic_to_shared(dcp_smem) +
-             (threadIdx.x >> 5) * (DCP_NIN * R * ROWB);
-  cols.ring = 0u;
+             (threadIdx.x >> 5) * (DCP_NIN * R * ROWB) + lane * 16;
+  cols.ring = cols.in = 0u;
+  const int vec = dcp_vec<CHECK>(it);
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int col = col0 + c;
     if (CHECK) cols.ring |= col < DCP_RX || col >= it.nx - DCP_RX ? 1u << c : 0u;
     cols.keep[c] = (unsigned)col < (unsigned)it.nx ? ~(typename DcpBits<T>::type)0 : 0;
-    if (CHECK && DCP_BC == DCP_BC_PERIODIC)
-      cols.pcol[c] = dcp_wrap(it.x0 - HX + lane + 32 * c, it.nx);
+    const int u = it.x0 - HX + (lane + 32 * c) * vec;  // first column of access c
+    cols.in |= (unsigned)u < (unsigned)it.nx ? 1u << c : 0u;
+    if (CHECK && DCP_BC == DCP_BC_PERIODIC) cols.pcol[c] = dcp_wrap(u, it.nx);
   }
   // Rows before the first streamed row count as zeros: exact ghosts above the
   // array; inside the array they only feed warm-up rows that are never written.
@@ -290,25 +310,46 @@ __device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Pro& pro, Out
 #pragma unroll
       for (int c = 0; c < C; ++c) st[l][d][c] = (T)0;
   int j = it.y0 - K * RY;
-  const int jend = it.y1 + K * RY;
-  int slot = 0;
+  const int jend = it.y1 + K * RY;   // rows j >= jout finish a written row
+  const int jout = it.y0 + K * RY;
+  unsigned so = 0;                   // ring offset of row j
   __syncwarp();  // the previous item's rows have been read
-  for (int r = 0; r < D; ++r) dcp_fetch_row<CHECK, false>(r, j + r, it, cols);
+  for (int r = 0; r < D; ++r) dcp_request_checked<CHECK>(r * ROWB, j + r, it, cols);
   // Rows [f0, f1] run without row tests: every row such an iteration touches
   // -- level rows from j - K*RY, the requested row j + D -- lies inside the
   // array and outside a fixed ring (periodic: the requested row).
   const int f0 = DCP_BC == DCP_BC_PERIODIC ? -D : K * RY + RING;
   const int f1 = min(jend - 1, it.ny - (DCP_BC == DCP_BC_PERIODIC ? 0 : RING) - 1 - D);
+  T a[C];
   while (j < jend) {
-    if (j >= f0) {
+    if (j >= f0 && j < f1) {
+      const T* src[DCP_NIN];
+      dcp_src<CHECK>(src, j + D, it);
+      long long gi = (long long)(j - K * RY) * it.nx + col0;  // the lane's first element of the finished row
 #pragma unroll 1
-      for (; j < f1; j += 2) {  // pairs: the partial sums alternate registers
-        dcp_iter<CHECK, true>(st, slot, j, it, cols, km, pro, output, guard);
-        dcp_iter<CHECK, true>(st, slot, j + 1, it, cols, km, pro, output, guard);
-      }
+      do {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // pairs: the partial sums alternate registers
+          dcp_wait_copies<D - 1>();  // this lane's copies of row j have landed
+          __syncwarp();              // every lane's have, and row j - 1 has been read
+          dcp_request<CHECK>((so - ROWB) & RMASK, src, cols.in, it, cols);
+#pragma unroll
+          for (int l = 0; l < DCP_NLOAD; ++l) src[l] += it.nx;
+          dcp_row<CHECK, true>(a, st, so, j, it, cols, km, pro, guard);
+          so = (so + ROWB) & RMASK;
+          if (j >= jout) output(gi, a);
+          gi += it.nx;
+          ++j;
+        }
+      } while (j < f1);
     }
     if (j < jend) {
-      dcp_iter<CHECK, false>(st, slot, j, it, cols, km, pro, output, guard);
+      dcp_wait_copies<D - 1>();
+      __syncwarp();
+      dcp_request_checked<CHECK>((so - ROWB) & RMASK, j + D, it, cols);
+      dcp_row<CHECK, false>(a, st, so, j, it, cols, km, pro, guard);
+      so = (so + ROWB) & RMASK;
+      if (j >= jout) output((long long)(j - K * RY) * it.nx + col0, a);
       ++j;
     }
   }
@@ -365,7 +406,6 @@ extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(co
   const int SEG = p.seg > 0 ? p.seg : ny;
   const int segs = (ny + SEG - 1) / SEG;
   const int items = strips * segs;
-  const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * DCP_THREADS + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * DCP_THREADS) >> 5;
   DcpGuard guard;
@@ -382,12 +422,10 @@ extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(co
     it.y0 = sg * SEG;
     it.y1 = min(ny, it.y0 + SEG);
     it.vec = 0;
-    const int col0 = it.x0 - HX + lane * C;
     const unsigned wm = dcp_written(it.x0, nx);
     dcp_stream(
         it, [&](const T (&ld)[DCP_NIN]) { return dcp_pro(ld, sc); }, guard, km,
-        [&](int y, const T (&v)[C]) {
-          const long long gi = (long long)y * nx + col0;
+        [&](long long gi, const T (&v)[C]) {
 #if DCP_POST
           T sv[DCP_ARR(DCP_NSTORE)][C];
 #pragma unroll
@@ -434,7 +472,6 @@ struct DcpBatchParams {
 };
 
 extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(const DcpBatchParams p) {
-  const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * DCP_THREADS + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * DCP_THREADS) >> 5;
   DcpGuard guard;
@@ -462,12 +499,12 @@ extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(co
                                    reinterpret_cast<unsigned long long>(I.out) |
                                    (unsigned long long)I.nx * sizeof(T);
     it.vec = (mis & 15) == 0 ? C : (C > 2 && (mis & 7) == 0 ? 2 : 1);
-    T* out = I.out + it.x0 - HX + lane * C;
-    const int nx = I.nx, vec = it.vec;
-    const unsigned wm = dcp_written(it.x0, nx);
+    T* out = I.out;
+    const int vec = it.vec;
+    const unsigned wm = dcp_written(it.x0, I.nx);
     dcp_stream(
         it, [&](const T (&ld)[DCP_NIN]) { return ld[0]; }, guard, km,
-        [&](int y, const T (&v)[C]) { dcp_write_row(out + (long long)y * nx, v, wm, vec); });
+        [&](long long gi, const T (&v)[C]) { dcp_write_row(out + gi, v, wm, vec); });
   }
 #if DCP_GUARD
   guard.flush(p.guard);
