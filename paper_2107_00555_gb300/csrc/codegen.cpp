@@ -96,7 +96,7 @@ std::string op_expr(int op, int dtype, double imm_v, const std::string& a, const
     case DCP_EXP: return (dtype == DCP_F64 ? "dcp_exp64(" : "dcp_exp(") + a + ")";
     case DCP_SIN: return (dtype == DCP_F64 ? "dcp_sin64(" : "dcp_sin(") + a + ")";
     case DCP_COS: return (dtype == DCP_F64 ? "dcp_cos64(" : "dcp_cos(") + a + ")";
-    case DCP_TANH: return "dcp_tanh(" + a + ")";
+    case DCP_TANH: return (dtype == DCP_F64 ? "dcp_tanh64(" : "dcp_tanh(") + a + ")";
     case DCP_SQRT: return "dcp_sqrt(" + a + ")";
     case DCP_SQUARE: return "dcp_square(" + a + ")";
     case DCP_ADD: return "dcp_add(" + a + ", " + b + ")";
@@ -227,7 +227,8 @@ uint64_t skeleton_hash(const std::string& body) {
       {"k_axis.cuh", kernel_axis_source()},
       {"k_math64.cuh", kernel_math64_source()},
       {"k_stencil_adj.cuh", kernel_adj_source()},
-      {"k_stencil2d_coop.cuh", kernel_coop_source()}};
+      {"k_stencil2d_coop.cuh", kernel_coop_source()},
+      {"k_tanh64.cuh", kernel_tanh64_source()}};
   unsigned used = 0;
   for (size_t i = 0; i < sizeof skel / sizeof skel[0]; ++i)
     if (body.find(std::string("#include \"") + skel[i].first + "\"") != std::string::npos) used |= 1u << i;
@@ -244,8 +245,8 @@ uint64_t skeleton_hash(const std::string& body) {
 }
 
 std::string finish(const std::string& prefix, const std::string& b) {
-  // binary64 exp / sin / cos come from k_math64.cuh; it is included only by
-  // kernels that call them, so other kernels' sources (and names) do not
+  // binary64 exp / sin / cos come from k_math64.cuh and tanh from
+  // k_tanh64.cuh; they are included only by kernels that call them, so other kernels' sources (and names) do not
   // depend on it
   std::string body = b;
   const std::string dev = "#include \"dcp_device.cuh\"\n";
@@ -254,6 +255,8 @@ std::string finish(const std::string& prefix, const std::string& b) {
                                   body.find("dcp_sin64(") != std::string::npos ||
                                   body.find("dcp_cos64(") != std::string::npos))
     body.insert(at + dev.size(), "#include \"k_math64.cuh\"\n");
+  if (at != std::string::npos && body.find("dcp_tanh64(") != std::string::npos)
+    body.insert(at + dev.size(), "#include \"k_tanh64.cuh\"\n");
   char name[64];
   std::snprintf(name, sizeof name, "%s_%016" PRIx64, prefix.c_str(),
                 fnv1a(body) ^ skeleton_hash(body));

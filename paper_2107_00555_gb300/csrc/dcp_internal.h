@@ -187,6 +187,8 @@ const char* kernel_stencil3d_source();  // k_stencil3d.cuh
 const char* kernel_stream_source();     // k_stencil2d_stream.cuh
 const char* kernel_axis_source();       // k_axis.cuh
 const char* kernel_math64_source();     // k_math64.cuh
+const char* kernel_tanh64_source();     // k_tanh64.cuh
+const char* kernel_tanh64_table_source();  // k_tanh64_table.cuh
 const char* kernel_adj_source();        // k_stencil_adj.cuh
 const char* kernel_coop_source();       // k_stencil2d_coop.cuh
 
