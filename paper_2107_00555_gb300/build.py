@@ -33,6 +33,7 @@ EMBED = [("dcp_device.cuh", "device_header_source"),
          ("k_stencil2d_stream.cuh", "kernel_stream_source"),
          ("k_axis.cuh", "kernel_axis_source"),
          ("k_math64.cuh", "kernel_math64_source"),
+         ("k_stencil3d_col.cuh", "kernel_column_source"),
          ("k_tanh64.cuh", "kernel_tanh64_source"),
          ("k_tanh64_table.cuh", "kernel_tanh64_table_source"),
          ("k_stencil_adj.cuh", "kernel_adj_source"),

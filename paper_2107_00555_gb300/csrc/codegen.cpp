@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <sstream>
@@ -228,7 +229,8 @@ uint64_t skeleton_hash(const std::string& body) {
       {"k_math64.cuh", kernel_math64_source()},
       {"k_stencil_adj.cuh", kernel_adj_source()},
       {"k_stencil2d_coop.cuh", kernel_coop_source()},
-      {"k_tanh64.cuh", kernel_tanh64_source()}};
+      {"k_tanh64.cuh", kernel_tanh64_source()},
+      {"k_stencil3d_col.cuh", kernel_column_source()}};
   unsigned used = 0;
   for (size_t i = 0; i < sizeof skel / sizeof skel[0]; ++i)
     if (body.find(std::string("#include \"") + skel[i].first + "\"") != std::string::npos) used |= 1u << i;
@@ -789,6 +791,155 @@ static void emit_stream_row(std::ostringstream& os, int T, int s, const Sum2& p,
   os << "  }\n};\n";
 }
 
+// Binary64 3-D stars on a deferred weight are summed by shared pairs (see
+// k_stencil3d_col.cuh) when the points at y +- 1 and z +- 1 have ratio 1 and
+// the others lie in the row (|dx| <= 1); every 3-D kernel form evaluates
+// D = north + below, then the row's points in listed order, then south +
+// above, so all forms round alike.  (Steps that apply their weights keep the
+// listed order: a pair would take two operations, and the planes form, which
+// runs their epilogues, does not share it.)
+struct Sum3 {
+  bool pairs = false;
+  int n = -1, s = -1, b = -1, t = -1;  // north, south, below (z - 1), above (z + 1)
+  std::vector<int> row;                // the row's points, listed order
+};
+
+Sum3 plan_sum3(int T, const std::vector<int32_t>& offs, const std::vector<double>& w, const Defer& df) {
+  Sum3 p;
+  if (T != DCP_F64 || !df.on) return p;
+  for (int k = 0; k < (int)w.size(); ++k) {
+    const int dz = offs[k * 3], dy = offs[k * 3 + 1], dx = offs[k * 3 + 2];
+    int* slot = dz == 0 && dy == -1 && dx == 0 ? &p.n
+                : dz == 0 && dy == 1 && dx == 0 ? &p.s
+                : dz == -1 && dy == 0 && dx == 0 ? &p.b
+                : dz == 1 && dy == 0 && dx == 0 ? &p.t : nullptr;
+    if (slot) {
+      if (*slot >= 0) return p;
+      *slot = k;
+    } else if (dz == 0 && dy == 0 && dx >= -1 && dx <= 1) {
+      for (int r : p.row)
+        if (offs[r * 3 + 2] == dx) return p;
+      p.row.push_back(k);
+    } else {
+      return p;
+    }
+  }
+  if (p.n < 0 || p.s < 0 || p.b < 0 || p.t < 0) return p;
+  p.pairs = df.ratio[p.n] == 1.0 && df.ratio[p.s] == 1.0 && df.ratio[p.b] == 1.0 && df.ratio[p.t] == 1.0;
+  return p;
+}
+
+// A row point of ratio r added to `acc`.
+std::string row_expr(int T, double r, const std::string& x, MulRegs& km) {
+  if (r == 1.0) return add_expr(T, x, "acc", km);
+  return "dcp_fma_rn(" + km.get(T, r) + ", " + x + ", acc)";
+}
+
+// Does a binary32 3-D star list its points as the column kernel adds them:
+// in-plane star points, then below, then above?
+bool listed_star3(const std::vector<int32_t>& offs, int n) {
+  if (n < 3) return false;
+  for (int k = 0; k < n; ++k) {
+    const int dz = offs[k * 3], dy = offs[k * 3 + 1], dx = offs[k * 3 + 2];
+    if (k == n - 1 ? !(dz == 1 && !dy && !dx)
+        : k == n - 2 ? !(dz == -1 && !dy && !dx)
+                     : (dz != 0 || std::abs(dy) + std::abs(dx) > 1))
+      return false;
+  }
+  return true;
+}
+
+// Warp-streamed columns of a 3-D star (k_stencil3d_col.cuh).
+static CodegenOut gen_column_kernel(const GraphImpl& g, const Group& G, int s0, int s1, int max_vec) {
+  NameScope names;
+  const int T = G.dtype, K = s1 - s0, C = stream_cols_per_lane(T);
+  const bool first = s0 == 0, last = s1 == (int)G.steps.size();
+  const bool f64 = T == DCP_F64;
+  int vec = std::min(C, max_vec);
+  while (G.shape.back() % vec != 0) vec /= 2;
+  std::ostringstream os;
+  os << "// dcp 3-D column stencil kernel: " << K << " steps per launch, bc " << G.bc << "\n";
+  os << "#define DCP_T " << dtype_cname(T) << "\n#define DCP_C " << C << "\n#define DCP_CY " << G.cy
+     << "\n#define DCP_LX " << G.lx << "\n#define DCP_NSTEPS " << K << "\n#define DCP_R " << kColumnRing << "\n#define DCP_W "
+     << column_width(G, K) << "\n#define DCP_VEC " << vec << "\n#define DCP_PAIRS " << (f64 ? 1 : 0)
+     << "\n#define DCP_BC " << G.bc << "\n#define DCP_THREADS " << G.threads << "\n#define DCP_LAST "
+     << (last ? 1 : 0) << "\n#define DCP_POST "
+     << (last && (!G.post.empty() || !G.reds.empty() || G.stores.size() != 1) ? 1 : 0)
+     << "\n#define DCP_MINB " << std::max(1, G.min_ctas) << "\n#define DCP_NSTORE "
+     << (last ? (int)G.stores.size() : 1) << "\n#define DCP_NRED " << (last ? (int)G.reds.size() : 0)
+     << "\n#define DCP_NSCALAR " << G.scalars.size() << "\n";
+  const Defer guard = first ? plan_defer(g, G, 0) : Defer();
+  os << "#define DCP_GUARD " << (guard.on ? 1 : 0) << "\n";
+  os << red_op_fn(g, last ? G.reds : std::vector<int>{});
+  os << "#include \"dcp_device.cuh\"\n";
+  emit_stencil_post(os, g, G, last);
+  const char* fn = "__device__ __forceinline__ DCP_T ";
+  const std::string kp = ", const DCP_T (&km)[DCP_NK])";
+  os << "template <int S> " << fn << "dcp_epi(DCP_T v);\n";
+  MulRegs km;
+  km.on = f64;
+  std::ostringstream sums, decl;
+  CodegenOut out;
+  for (int s = 0; s < K; ++s) {
+    const StepDesc& sd = G.steps[s0 + s];
+    const Node& sn = g.nodes[sd.node];
+    const Defer df = plan_defer(g, G, s0 + s);
+    const std::string sp = "template <> " + std::string(fn);
+    const std::string id = "<" + std::to_string(s) + ">";
+    auto side = [&](int dx) { return dx < 0 ? "l" : (dx > 0 ? "r" : "c"); };
+    if (f64) {
+      const Sum3 p = plan_sum3(T, G.offsets, sn.weights, df);
+      sums << "// deferred common weight: the ratios w_k / f\n";
+      for (int c = 0; c < C; ++c) {
+        const std::string ic = "<" + std::to_string(s) + ", " + std::to_string(c) + ">";
+        sums << sp << "dcp_d" << ic << "(DCP_T up, DCP_T before" << kp << " {\n  (void)km;\n  return "
+             << add_expr(T, "up", "before", km) << ";\n}\n";
+        sums << sp << "dcp_in" << ic << "(DCP_T d, DCP_T c, DCP_T l, DCP_T r" << kp
+             << " {\n  (void)km; (void)c; (void)l; (void)r;\n  DCP_T acc = d;\n";
+        for (int k : p.row)
+          sums << "  acc = " << row_expr(T, df.ratio[k], side(G.offsets[k * 3 + 2]), km) << ";\n";
+        sums << "  return acc;\n}\n";
+        sums << sp << "dcp_fin" << ic << "(DCP_T acc, DCP_T d" << kp << " {\n  (void)km;\n  acc = "
+             << add_expr(T, "d", "acc", km) << ";\n";
+        if (df.scale != 1.0) sums << "  acc = dcp_mul_rn(" << weight_literal(T, df.scale) << ", acc);\n";
+        sums << "  return acc;\n}\n";
+      }
+      if (s == 0)
+        decl << "template <int S, int I> " << fn << "dcp_d(DCP_T up, DCP_T before" << kp
+             << ";\ntemplate <int S, int I> " << fn << "dcp_in(DCP_T d, DCP_T c, DCP_T l, DCP_T r" << kp
+             << ";\ntemplate <int S, int I> " << fn << "dcp_fin(DCP_T acc, DCP_T d" << kp << ";\n";
+    } else {
+      sums << sp << "dcp_in" << id << "(DCP_T c, DCP_T l, DCP_T r, DCP_T up, DCP_T dn, DCP_T before) {\n"
+           << "  (void)c; (void)l; (void)r; (void)up; (void)dn;\n";
+      const int n = sn.npts();
+      for (int k = 0; k + 1 < n; ++k) {
+        const int dz = G.offsets[k * 3], dy = G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
+        const std::string x = dz ? "before" : (dy < 0 ? "up" : (dy > 0 ? "dn" : side(dx)));
+        emit_term(sums, T, "acc", x, sn.weights[k], k == 0, false, km);
+      }
+      sums << "  return acc;\n}\n";
+      sums << sp << "dcp_fin" << id << "(DCP_T acc, DCP_T c) {\n";
+      emit_term(sums, T, "acc", "c", sn.weights[n - 1], false, false, km);
+      sums << "  return acc;\n}\n";
+      if (s == 0)
+        decl << "template <int S> " << fn
+             << "dcp_in(DCP_T c, DCP_T l, DCP_T r, DCP_T up, DCP_T dn, DCP_T before);\ntemplate <int S> " << fn
+             << "dcp_fin(DCP_T acc, DCP_T c);\n";
+    }
+    if (df.on) out.defer_scales.push_back(df.scale);
+    sums << sp << "dcp_epi" << id << "(DCP_T v) {\n" << epi_body(g, sd) << "}\n";
+  }
+  os << km.table() << decl.str() << sums.str();
+  os << "#include \"k_stencil3d_col.cuh\"\n";
+  out.threads = G.threads;
+  out.vec = vec;
+  out.guard_max_input = guard.on ? guard.max_input : 0.0;
+  out.smem_bytes = G.threads / 32 * kColumnRing * (32 / G.lx * G.cy + 2 * K) * ((G.lx + 2) * C) * dtype_size(T);
+  out.source = finish("dcp_col3d", os.str());
+  out.name = kname_of(out.source);
+  return out;
+}
+
 // Warp-stream form (k_stencil2d_stream.cuh) of a 1-D / 2-D stencil launch.
 static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, int s1, int max_vec) {
   NameScope names;
@@ -880,6 +1031,7 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
 
 CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1, int max_vec) {
   if (G.variant == 1) return gen_stream_kernel(g, G, s0, s1, max_vec);
+  if (G.variant == 3) return gen_column_kernel(g, G, s0, s1, max_vec);
   NameScope names;
   const bool batch = G.kind == GroupKind::Batch;
   const int nd = batch ? 2 : (int)G.shape.size();
@@ -980,15 +1132,28 @@ CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1
     auto wt = [&](int k) { return df.on ? df.ratio[k] : sn.weights[k]; };
     if (df.on) sums << "  // deferred common weight: the ratios w_k / f\n";
     if (df.on) out.defer_scales = {df.scale};
-    if (CX == 1) {
-      for (int i = 0; i < sn.npts(); ++i) {
-        const int k = order[i];
-        int dz = G.offsets[k * 3], dy = G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
-        std::string x = "pl[" + std::to_string(dz + rz) + "][c + (" + std::to_string(dy * PW + dx) + ")]";
-        emit_term(sums, T, "acc", x, wt(k), i == 0, df.on, km);
+    const Sum3 p3 = plan_sum3(T, G.offsets, sn.weights, df);
+    // the weighted sum of one cell; x(k) names point k's value
+    auto emit_cell = [&](const std::string& a, const std::function<std::string(int)>& x) {
+      if (p3.pairs) {
+        sums << "  DCP_T " << a << ";\n  {\n  DCP_T acc = " << add_expr(T, x(p3.n), x(p3.b), km)
+             << ";\n";
+        for (int k : p3.row) sums << "  acc = " << row_expr(T, df.ratio[k], x(k), km) << ";\n";
+        sums << "  const DCP_T d2 = " << add_expr(T, x(p3.t), x(p3.s), km) << ";\n  " << a
+             << " = " << add_expr(T, "d2", "acc", km) << ";\n  }\n";
+      } else {
+        for (int i = 0; i < sn.npts(); ++i)
+          emit_term(sums, T, a, x(order[i]), wt(order[i]), i == 0, df.on, km);
       }
-      if (df.scale != 1.0) sums << "  acc = dcp_mul_rn(" << weight_literal(T, df.scale) << ", acc);\n";
-      sums << "  v[0] = acc;\n";
+      if (df.scale != 1.0)
+        sums << "  " << a << " = dcp_mul_rn(" << weight_literal(T, df.scale) << ", " << a << ");\n";
+    };
+    if (CX == 1) {
+      emit_cell("a0", [&](int k) {
+        int dz = G.offsets[k * 3], dy = G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
+        return "pl[" + std::to_string(dz + rz) + "][c + (" + std::to_string(dy * PW + dx) + ")]";
+      });
+      sums << "  v[0] = a0;\n";
     } else {
       // one aligned pair load per distinct (plane, pair index) the two cells read
       auto floor_div2 = [](int o) { return o >= 0 ? o / 2 : -((-o + 1) / 2); };
@@ -1007,16 +1172,12 @@ CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1
         }
       for (int j = 0; j < 2; ++j) {
         std::string a = "a" + std::to_string(j);
-        for (int i = 0; i < sn.npts(); ++i) {
-          const int k = order[i];
+        emit_cell(a, [&](int k) {
           int dz = G.offsets[k * 3], dy = G.offsets[k * 3 + 1], dx = G.offsets[k * 3 + 2];
           int o = dy * PW + dx + j, q = floor_div2(o);
-          std::string x = pairs[std::make_pair(dz + rz, q)] + (o - 2 * q == 0 ? ".x" : ".y");
-          emit_term(sums, T, a, x, wt(k), i == 0, df.on, km);
-        }
-        if (df.scale != 1.0)
-          sums << "  " << a << " = dcp_mul_rn(" << weight_literal(T, df.scale) << ", " << a << ");\n";
-        sums << "  v[" << j << "] = a" << j << ";\n";
+          return pairs[std::make_pair(dz + rz, q)] + (o - 2 * q == 0 ? ".x" : ".y");
+        });
+        sums << "  v[" << j << "] = " << a << ";\n";
       }
     }
     sums << "}\n";
@@ -1029,6 +1190,18 @@ CodegenOut gen_stencil_kernel(const GraphImpl& g, const Group& G, int s0, int s1
                       os.str());
   out.name = kname_of(out.source);
   return out;
+}
+
+bool column_eligible(const GraphImpl& g, const Group& G) {
+  if (G.kind != GroupKind::Stencil || G.shape.size() != 3 || !G.members.empty()) return false;
+  if (G.radius[0] != 1 || G.radius[1] > 1 || G.radius[2] > 1) return false;
+  for (int s = 0; s < (int)G.steps.size(); ++s) {
+    const Node& n = g.nodes[G.steps[s].node];
+    if (G.dtype == DCP_F64 ? !plan_sum3(G.dtype, G.offsets, n.weights, plan_defer(g, G, s)).pairs
+                           : !listed_star3(G.offsets, n.npts()))
+      return false;
+  }
+  return true;
 }
 
 CodegenOut gen_batch_kernel(const GraphImpl& g, const Group& G, int s0, int s1) {

@@ -143,8 +143,10 @@ struct Group {
   int threads = 256;
   int blocks_per_sm = 4;
   int variant = 0;              // stencils: 0 = shared-memory tile, 1 = warp stream,
-                                //           2 = cooperative (every step in one launch)
-  int seg = 0;                  // warp stream: rows per work item (single arrays)
+                                //           2 = cooperative (every step in one launch),
+                                //           3 = 3-D warp-streamed columns
+  int seg = 0;                  // warp stream: rows per work item; columns: planes per work item
+  int cy = 1, lx = 32;          // 3-D columns: rows per lane, lanes along x
   int prefetch = 1;             // warp stream: rows requested ahead, in row windows (2*ry+1)
   int min_ctas = 0;             // warp stream: CTAs per SM the register budget must allow (0: any)
   int cx = 1;                   // 3-D stencils: cells per thread along x (1 or 2)
@@ -187,6 +189,7 @@ const char* kernel_stencil3d_source();  // k_stencil3d.cuh
 const char* kernel_stream_source();     // k_stencil2d_stream.cuh
 const char* kernel_axis_source();       // k_axis.cuh
 const char* kernel_math64_source();     // k_math64.cuh
+const char* kernel_column_source();     // k_stencil3d_col.cuh
 const char* kernel_tanh64_source();     // k_tanh64.cuh
 const char* kernel_tanh64_table_source();  // k_tanh64_table.cuh
 const char* kernel_adj_source();        // k_stencil_adj.cuh
@@ -286,6 +289,17 @@ inline int stream_width(const Group& G, int nsteps) {
   return (32 * C - (h + C - 1) / C * C - h) / C * C;
 }
 bool stream_eligible(const Group& G, int depth);
+// 3-D columns: planes of a warp's ring, columns written per warp in a launch
+// of nsteps steps, and whether the group's steps take the form
+constexpr int kColumnRing = 3;
+inline int column_width(const Group& G, int nsteps) {
+  const int C = stream_cols_per_lane(G.dtype);
+  return G.lx * C - (nsteps > 1 ? 2 * C : 0);
+}
+// CTAs (of one warp) per SM its registers must allow: two warps per scheduler
+// for eight binary64 rows per lane, three otherwise
+inline int column_min_ctas(const Group& G) { return G.dtype == DCP_F64 && G.cy == 8 ? 8 : 12; }
+bool column_eligible(const GraphImpl& g, const Group& G);
 // can the cooperative form run this group with a ty x tx tile (steps <= 63,
 // 1-D / 2-D, each ragged edge tile at least a radius wide)?
 bool coop_eligible(const Group& G, int ty, int tx);

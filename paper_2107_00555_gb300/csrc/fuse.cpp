@@ -629,13 +629,101 @@ struct Planner {
     return t;
   }
 
+  // 3-D stars without a prologue run as warp-streamed columns where those are
+  // faster, unless a tile option asks for the shared-memory planes: binary64
+  // one step per launch, binary32 two.  A warp (nw per scheduler) streams seg + 2 K planes, one
+  // plane costing the larger of its latency and the issue (binary32, about 9
+  // instructions per cell and level) or FP64 pipe time (64 cycles per
+  // operation of the warp) of the scheduler's warps.
+  void choose_columns(Group& G) {
+    G.variant = 0;
+    const auto has = [&](int key) { return g.options.count(key) > 0; };
+    if (!column_eligible(g, G) || has(DCP_OPT_TILE_X) || has(DCP_OPT_TILE_Y) || has(DCP_OPT_TILE_Z) ||
+        has(DCP_OPT_CELLS_PER_THREAD) || G.shape[0] * G.shape[1] * G.shape[2] == 0 ||
+        G.shape[1] * G.shape[2] > 0x7fffffff)  // (offsets within a plane are 32-bit)
+      return;
+    const bool f64 = G.dtype == DCP_F64;
+    const int S = (int)G.steps.size();
+    int kmax = f64 || !(flags & DCP_TIME_TILE) ? 1 : 2;
+    kmax = std::min<int64_t>({kmax, S, std::max<int64_t>(1, opt(DCP_OPT_TIME_TILE_DEPTH, 2))});
+    const int64_t nz = G.shape[0], ny = G.shape[1], nx = G.shape[2];
+    double epi = 0;
+    for (const StepDesc& st : G.steps)
+      for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
+    epi /= S;
+    const int pts = (int)G.offsets.size() / 3;
+    const double bytes = 2.0 * nz * ny * nx * dtype_size(G.dtype);
+    const double mem = bytes / (bytes > 100e6 ? 3237.0 : 6500.0);
+    // measured over the counted cycles (512^3, 256^3, 300 x 333 x 381)
+    const double busy = G.bc == DCP_BC_PERIODIC ? 1.15 : 1.09;
+    int bcy = 4, blx = 32;
+    int64_t bseg = 1;
+    // the shared-memory planes: whole tiles of 8 x 32 cells, one operation more
+    double best = 1e300;
+    if (f64) {
+      const double padded = (double)nz * ((ny + 7) / 8 * 8) * ((nx + 31) / 32 * 32);
+      best = 0.95 * (std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / 304 + 3000) + 6200) * S;
+    }
+    const int lx0 = G.lx, cy0 = G.cy;
+    bool column = !f64;
+    for (int K = 1; K <= kmax; ++K)
+      for (int lx : {32, 16})
+        for (int cy : {8, 4, 2}) {
+          if (!f64 && (cy == 8 || lx != 32)) continue;
+          G.lx = lx;
+          const int rows_w = 32 / lx * cy;  // rows per warp
+          if (rows_w > 2 && rows_w / 2 >= ny) continue;
+          const int64_t strips = (nx + column_width(G, K) - 1) / column_width(G, K);
+          const int64_t blocks = (ny + rows_w - 1) / rows_w;
+          const double rows = K == 1 ? cy : 2 * cy + 2;  // rows summed per plane, all levels
+          const double issue = f64 ? cy * (2 * 64 * (pts - 3 + (cy + 1.0) / cy) + epi) + 100
+                                   : rows * (4.0 * pts + 10 + epi) + (cy + 2 * K) * 9 + 60;
+          const double latency = f64 ? 1500 : 500.0 * K + 300;
+          const double ends = f64 ? 0.5 : 2.0 * K;  // planes an item pays for beside its own
+          // warps per scheduler: what the registers of the form allow without
+          // spills (512^3 binary64, 8 rows per lane: 1.22 ms per step at 2,
+          // 1.41 at 3; 300 x 333 x 381 binary32: 59 us at 3, 72 at 4)
+          const int nmax = f64 && cy == 8 ? 2 : 3;
+          for (int n = 1; n <= nmax; ++n)
+            for (int wv = 1; wv <= 16; ++wv) {  // items in whole waves of n warps per scheduler
+              const int64_t segs = (int64_t)wv * n * 608 / (strips * blocks);
+              if (segs < 1) continue;
+              const int64_t sg = (nz + std::min(segs, nz) - 1) / std::min(segs, nz);
+              const int64_t items = strips * blocks * ((nz + sg - 1) / sg);
+              const int64_t per = (items + 607) / 608;
+              const int64_t waves = (per + n - 1) / n;
+              // (one warp alone keeps its scheduler's FP64 pipe busy 70 % of the time)
+              const int64_t nn = std::min<int64_t>(per, n);
+              const double c = (std::max(mem, waves * (double)(sg + ends) *
+                                                  std::max(latency, issue * nn * busy * (f64 && nn == 1 ? 1.3 : 1.0))) +
+                                6200) * ((S + K - 1) / K);
+              if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
+              if (segs >= nz) break;
+            }
+          if (strips * blocks > 16 * nmax * 608) {  // wide grids: long columns
+            const int64_t sg = std::min<int64_t>(nz, 64);
+            const double c = ((double)strips * blocks * nz / sg / 608 * (sg + ends) * issue + 6200) * ((S + K - 1) / K);
+            if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
+          }
+        }
+    G.lx = lx0;
+    G.cy = cy0;
+    if (!column) return;
+    G.cy = bcy;
+    G.lx = blx;
+    G.seg = (int)bseg;
+    G.variant = 3;
+    G.threads = 32;
+    G.min_ctas = column_min_ctas(G);
+  }
+
   // Kernel form, depth, rows per work item or tile of a 1-D / 2-D stencil
   // group, each unless an option sets it.
   void choose_stencil_tiling(Group& G) {
     choose_stencil_tiling_impl(G);
     const int nd = G.kind == GroupKind::Batch ? 2 : (int)G.shape.size();
     if (nd == 3) {
-      G.variant = 0;
+      choose_columns(G);
       return;
     }
     const auto has = [&](int key) { return g.options.count(key) > 0; };

@@ -71,11 +71,11 @@ CubinRef nvrtc_compile(const std::string& src, const std::string& name, double* 
   const char* hdr_src[] = {device_header_source(), kernel_map_source(), kernel_stencil2d_source(),
                            kernel_stencil3d_source(), kernel_stream_source(), kernel_axis_source(),
                            kernel_math64_source(), kernel_adj_source(), kernel_coop_source(),
-                           kernel_tanh64_source(), kernel_tanh64_table_source()};
+                           kernel_tanh64_source(), kernel_tanh64_table_source(), kernel_column_source()};
   const char* hdr_name[] = {"dcp_device.cuh", "k_map.cuh", "k_stencil2d.cuh", "k_stencil3d.cuh",
                             "k_stencil2d_stream.cuh", "k_axis.cuh", "k_math64.cuh",
                             "k_stencil_adj.cuh", "k_stencil2d_coop.cuh", "k_tanh64.cuh",
-                            "k_tanh64_table.cuh"};
+                            "k_tanh64_table.cuh", "k_stencil3d_col.cuh"};
   nvrtcProgram prog;
   nvrtcResult r = nvrtcCreateProgram(&prog, src.c_str(), (name + ".cu").c_str(),
                                      (int)(sizeof hdr_src / sizeof hdr_src[0]), hdr_src,

@@ -574,8 +574,9 @@ static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const
   CUfunction fn = ls.fn;
   int occ = ls.occupancy;
   int64_t gx;
-  if (G.variant == 1) {
-    // warp stream: one warp per (strip, row segment) work item, warps stride
+  if (G.variant == 1 || G.variant == 3) {
+    // warp stream: one warp per (strip, row segment) work item, columns: per
+    // (strip, rows, planes); warps stride
     // the kernel's access width suits the row length; buffers off its boundary
     // take the element-wise variant
     uintptr_t mis = 0;
@@ -589,8 +590,10 @@ static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const
       fn = ls.fn_scalar;
       occ = ls.occ_scalar;
     }
-    const int W = stream_width(G, ls.s1 - ls.s0);
-    int64_t items = (int64_t)((p.nx + W - 1) / W) * ((p.ny + G.seg - 1) / G.seg);
+    const int W = G.variant == 1 ? stream_width(G, ls.s1 - ls.s0) : column_width(G, ls.s1 - ls.s0);
+    int64_t items = (int64_t)((p.nx + W - 1) / W);
+    if (G.variant == 1) items *= (p.ny + G.seg - 1) / G.seg;
+    else items *= (int64_t)((p.ny + 32 / G.lx * G.cy - 1) / (32 / G.lx * G.cy)) * ((p.nz + G.seg - 1) / G.seg);
     const int wpb = ls.code.threads / 32;
     int64_t warps = std::min<int64_t>(items, (int64_t)rt.sms * occ * wpb);
     gx = std::max<int64_t>(1, (warps + wpb - 1) / wpb);
@@ -871,6 +874,9 @@ std::vector<TuneCfg> tune_candidates(const Group& G, int sms) {
   const int S = (int)G.steps.size();
   const int nd = group_nd(G);
   if (nd == 3) {
+    // the planner's columns (tz slot = -3: rows per lane, planes per item,
+    // lanes along x)
+    if (G.variant == 3) c.push_back({G.depth, -3, G.cy, G.seg, G.lx});
     // one cell per thread (256-thread tiles) and paired cells along x
     const std::array<int, 3> tiles[] = {{32, 8, 32}, {64, 8, 32}, {16, 8, 32},
                                         {32, 4, 64}, {32, 16, 32}, {64, 4, 64}};
@@ -881,6 +887,9 @@ std::vector<TuneCfg> tune_candidates(const Group& G, int sms) {
       for (const auto& t : pair_tiles) c.push_back({1, t[0], t[1], t[2], 2});
     return c;
   }
+  // the planner's own choice
+  if (G.variant == 1) c.push_back({G.depth, -1, G.seg, G.prefetch, std::max(1, G.min_ctas)});
+  else if (G.variant == 0) c.push_back({G.depth, 1, G.tile[1], G.tile[2], 1});
   std::vector<int> depths;
   for (int d : {1, 2, 3, 4, 5, 8, 10})
     if (d <= S) depths.push_back(d);
@@ -947,7 +956,14 @@ std::vector<TuneCfg> tune_candidates(const Group& G, int sms) {
 void apply_config(GraphImpl& g, int gi, const TuneCfg& cfg) {
   Group& G = g.groups[gi];
   G.depth = cfg[0];
-  G.variant = cfg[1] == -1 ? 1 : (cfg[1] == -2 ? 2 : 0);
+  G.variant = cfg[1] == -1 ? 1 : (cfg[1] == -2 ? 2 : (cfg[1] == -3 ? 3 : 0));
+  if (G.variant == 3) {
+    G.cy = cfg[2];
+    G.seg = cfg[3];
+    G.lx = cfg[4];
+    G.min_ctas = column_min_ctas(G);
+    G.threads = 32;
+  }
   G.tile[0] = cfg[1] < 0 ? 1 : cfg[1];
   G.tile[1] = cfg[2];
   G.tile[2] = cfg[3];
@@ -967,7 +983,7 @@ void apply_config(GraphImpl& g, int gi, const TuneCfg& cfg) {
                                                    8 * G.depth * std::max(1, G.radius[1]));
       G.seg = (int)std::min<int64_t>(std::max<int64_t>(seg, 1), std::max<int64_t>(ny, 1));
     }
-  } else {
+  } else if (G.variant != 3) {
     G.threads = group_nd(G) == 3 || cfg[4] < 32 ? 256 : cfg[4];
   }
   std::vector<LaunchSpec> L = build_group_launches(g, gi);
@@ -1249,9 +1265,13 @@ std::string describe_plan(const GraphImpl& g) {
     if (G.kind == GroupKind::AxisReduce) os << ", \"axis\": " << G.axis;
     if (G.kind == GroupKind::Stencil && G.shape.size() == 3) os << ", \"cells_per_thread\": " << G.cx;
     if (G.kind != GroupKind::Map && G.kind != GroupKind::AxisReduce && G.kind != GroupKind::AdjTile)
-      os << ", \"kernel_form\": \"" << (G.variant == 1 ? "stream" : (G.variant == 2 ? "coop" : "tile")) << "\", \"seg\": " << G.seg
+      os << ", \"kernel_form\": \"" << (G.variant == 1 ? "stream" : (G.variant == 2 ? "coop" : (G.variant == 3 ? "column" : "tile"))) << "\", \"seg\": " << G.seg
          << ", \"prefetch\": " << G.prefetch << ", \"threads\": " << G.threads
          << ", \"min_ctas\": " << G.min_ctas;
+    if (G.kind == GroupKind::Stencil && G.variant == 3)
+      os << ", \"rows_per_lane\": " << G.cy << ", \"lanes_x\": " << G.lx;
+    if (G.kind == GroupKind::Stencil && G.variant == 3)
+      os << ", \"rows_per_lane\": " << G.cy << ", \"lanes_x\": " << G.lx;
     int epi = 0;
     for (const StepDesc& s : G.steps) epi += (int)s.epi.size();
     if (G.kind == GroupKind::AdjTile)
