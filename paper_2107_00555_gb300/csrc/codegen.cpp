@@ -320,7 +320,10 @@ CodegenOut gen_axis_kernel(const GraphImpl& g, const Group& G, bool vec_ok) {
   // the reduction tree's shared memory stays within 32 KB
   const int axmode = inner > 1 ? 0 : 1;
   int vec = vec_ok ? 16 / dtype_size(T) : 1;
-  if ((axmode == 0 ? inner : R) % vec != 0 || (int)G.reds.size() * vec > 16) vec = 1;
+  // (rows shorter than four vectors per thread of a warp gain nothing from
+  // unaligned ends)
+  if ((axmode == 0 ? inner : R) % vec != 0 && (axmode == 0 || R < 4 * 32 * vec)) vec = 1;
+  if ((int)G.reds.size() * vec > 16) vec = 1;
   os << "// dcp axis reduction kernel: " << G.members.size() << " prologue ops, " << G.loads.size()
      << " loads, " << G.reds.size() << " reductions along axis " << G.axis << "\n";
   os << "#define DCP_T " << dtype_cname(T) << "\n#define DCP_THREADS " << G.threads
@@ -765,23 +768,28 @@ static void emit_stream_row(std::ostringstream& os, int T, int s, const Sum2& p,
         if (offs[i * 3 + 1] < dy) started = true;
         if (offs[i * 3 + 1] == dy) pts.push_back(i);
       }
-      for (int c = 0; c < C; ++c) {
-        const std::string dst = k == 0 ? at("out", c) : st(k - 1, c);
-        const std::string src = k < 2 * ry ? st(k, c) : std::string("0");
-        bool fresh = !started;
-        const bool ring_sel = dy >= 0 && ry > 0;  // a ring cell's sum is its own value
-        os << "  {\n  DCP_T t = " << (started ? src : "(DCP_T)0") << ";\n";
-        for (int i : pts) {
+      // (term by term over the columns: neighbouring operations independent)
+      const bool ring_sel = dy >= 0;  // a ring cell's sum is its own value
+      auto src = [&](int c) { return k < 2 * ry ? st(k, c) : std::string("(DCP_T)0"); };
+      os << "  {\n  DCP_T t[" << C << "];\n";
+      if (started || pts.empty())
+        for (int c = 0; c < C; ++c) os << "  t[" << c << "] = " << (started ? src(c) : "(DCP_T)0") << ";\n";
+      bool fresh = !started;
+      for (int i : pts) {
+        for (int c = 0; c < C; ++c) {
           const int cc = c + offs[i * 3 + 2];
           const std::string x = cc < 0 ? at("lf", rx + cc) : (cc >= C ? at("rt", cc - C) : at("a", cc));
-          emit_row_term(os, T, "t", "t", x, p.w[i], fresh, p.df.on, km);
-          fresh = false;
+          emit_row_term(os, T, at("t", c), at("t", c), x, p.w[i], fresh, p.df.on, km);
         }
-        if (ring_sel || ry == 0)
-          os << "  if (RINGM && ((rm[" << k << "] >> " << c << ") & 1u)) t = "
-             << (dy == 0 ? at("a", c) : src) << ";\n";
-        os << "  " << dst << " = t;\n  }\n";
+        fresh = false;
       }
+      for (int c = 0; c < C; ++c) {
+        if (ring_sel)
+          os << "  if (RINGM && ((rm[" << k << "] >> " << c << ") & 1u)) t[" << c << "] = "
+             << (dy == 0 ? at("a", c) : src(c)) << ";\n";
+        os << "  " << (k == 0 ? at("out", c) : st(k - 1, c)) << " = t[" << c << "];\n";
+      }
+      os << "  }\n";
     }
   }
   if (p.df.scale != 1.0)

@@ -288,6 +288,9 @@ inline int stream_width(const Group& G, int nsteps) {
   const int C = stream_cols_per_lane(G.dtype), h = nsteps * G.radius[2];
   return (32 * C - (h + C - 1) / C * C - h) / C * C;
 }
+inline int default_stream_threads(const Group& G) {
+  return G.dtype == DCP_F64 && G.kind != GroupKind::Batch ? 64 : 32;
+}
 bool stream_eligible(const Group& G, int depth);
 // 3-D columns: planes of a warp's ring, columns written per warp in a launch
 // of nsteps steps, and whether the group's steps take the form

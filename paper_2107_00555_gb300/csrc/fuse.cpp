@@ -22,6 +22,7 @@
 //    connected components of Sec. 2.4 state fusion).
 #include <algorithm>
 #include <cmath>
+#include <map>
 #include <set>
 #include <sstream>
 
@@ -36,6 +37,7 @@ struct Planner {
   uint32_t flags;
   std::vector<std::vector<int>> users;
   std::vector<char> live, is_out;
+  std::map<int, int> axis_map;  // map planned into an axis-reduce group before its turn
 
   std::vector<Group>& batch_store;
   Planner(GraphImpl& gi, uint32_t f) : g(gi), flags(f), batch_store(gi.batch_store) {}
@@ -113,8 +115,35 @@ struct Planner {
     finalize();
   }
 
+  // Maps reached from value m that may join the prologue of reductions along
+  // `axis` of the group that will replace map group gi: same space, read only
+  // by such maps or by reductions along that axis, every operand computed
+  // there or before.  Collects them in `maps` and the reductions in nred.
+  bool axis_closure(int m, const Group& M, int gi, int axis, std::set<int>& maps, std::set<int>& reds) const {
+    for (int u : users[m]) {
+      if (!live[u] || in_vec(M.members, u) || maps.count(u)) continue;
+      const Node& un = g.nodes[u];
+      if (un.kind == Kind::Reduce && un.axis == axis) {
+        reds.insert(u);
+        continue;
+      }
+      if (un.kind != Kind::Map || un.shape != M.shape || is_out[u]) return false;
+      maps.insert(u);
+      if (!axis_closure(u, M, gi, axis, maps, reds)) return false;
+    }
+    return true;
+  }
+
   void plan_map(int v) {
     const Node& n = g.nodes[v];
+    auto planned = axis_map.find(v);
+    if (planned != axis_map.end()) {  // fused into an axis reduction's prologue
+      Group& G = g.groups[planned->second];
+      G.members.push_back(v);
+      g.value_group[v] = planned->second;
+      for (int a : n.in) add_operand(G, planned->second, a);
+      return;
+    }
     // (1) stencil step epilogue: a unary / immediate map of a stencil group's
     //     current output, which nothing else reads.
     if (fsub() && (op_is_unary(n.op) || op_is_scalar_imm(n.op))) {
@@ -220,20 +249,34 @@ struct Planner {
     R.shape = an.shape;
     R.axis = n.axis;
     bool absorbed = false;
+    std::set<int> later;
     if (fsub() && gi >= 0 && gi == (int)g.groups.size() - 1 &&
         g.groups[gi].kind == GroupKind::Map && computed_in(gi, a)) {
       const Group& M = g.groups[gi];
       bool ok = M.reds.empty() && M.shape == an.shape;
-      int nred = 0;
+      std::set<int> reds;
       for (int m : M.members) {
         if (is_out[m] || g.nodes[m].kind != Kind::Map) ok = false;
-        for (int u : users[m]) {
-          if (!live[u] || in_vec(M.members, u)) continue;
-          const Node& un = g.nodes[u];
-          if (un.kind == Kind::Reduce && un.axis == n.axis) ++nred;
-          else ok = false;
-        }
+        ok = ok && axis_closure(m, M, gi, n.axis, later, reds);
       }
+      // the operands of the maps still to come, and the limits of one kernel
+      std::set<int> loads(M.loads.begin(), M.loads.end()), scalars(M.scalars.begin(), M.scalars.end());
+      for (int u : later)
+        for (int b : g.nodes[u].in) {
+          if (in_vec(M.members, b) || later.count(b)) continue;
+          const bool known = g.nodes[b].kind == Kind::Input || (g.value_group[b] >= 0 && g.value_group[b] < gi);
+          ok = ok && known;
+          (g.nodes[b].shape.empty() ? scalars : loads).insert(b);
+        }
+      const int nred = (int)reds.size();
+      // binary64 maps with exp, sin and the like are bound by the FP64 pipe,
+      // which the map kernel keeps busier than a row tree: maps still to come
+      // then stay in its one pass (8063 x 140 binary64 columns 99 us against
+      // 168 in one kernel, 6751 x 1810 rows 784 against 848)
+      double cost = 0;
+      for (int m : M.members) cost += op_cycles(g.nodes[m].op, an.dtype);
+      if (an.dtype == DCP_F64 && !later.empty() && cost > 12 * op_cycles(DCP_ADD, DCP_F64)) ok = false;
+      if ((int)loads.size() > kMaxIO || (int)scalars.size() > kMaxIO) ok = false;
       if (ok && nred <= kMaxIO) {
         R.members = M.members;
         R.loads = M.loads;
@@ -248,6 +291,8 @@ struct Planner {
     int ri = (int)g.groups.size() - 1;
     g.value_group[v] = ri;
     for (int m : R.members) g.value_group[m] = ri;
+    if (absorbed)
+      for (int u : later) axis_map[u] = ri;
   }
 
   void plan_reduce(int v) {
@@ -529,6 +574,17 @@ struct Planner {
     return 4 * n;
   }
 
+  // FP64 operations per cell of a 2-D step: a run on its deferred weight
+  // shares the pairs of a 5-point star (two operations fewer).
+  double step_ops64(const Group& G) const {
+    const int pts = (int)G.offsets.size() / 3;
+    const Node& n = g.nodes[G.steps[0].node];
+    auto opt_on = g.options.find(DCP_OPT_DEFERRED_WEIGHT);
+    const bool run = G.steps.size() > 1 && G.steps[0].epi.empty() && defer_chunk_steps(n) > 0 &&
+                     (opt_on == g.options.end() || opt_on->second != 0);
+    return run ? std::max(1, pts == 5 ? pts - 2 : pts - 1) : pts;
+  }
+
   // Cycles of one launch of K steps of the warp-stream kernel, and the rows
   // per work item that give them: nw warps per scheduler (4 per SM) stream
   // seg + 2 K ry rows each, a row taking the larger of its latency and the
@@ -545,7 +601,7 @@ struct Planner {
     const int pts = (int)G.offsets.size() / 3;
     double issue, latency;
     if (G.dtype == DCP_F64) {
-      issue = K * 2.0 * 64 * std::max(2, pts - 1) + 60;
+      issue = K * 2.0 * 64 * step_ops64(G) + 60;
       latency = 300.0 + 500.0 * K;
     } else {
       issue = K * (7.0 + 4.0 * pts) + 42;
@@ -569,7 +625,10 @@ struct Planner {
       const int64_t items = strips * ((ny + sg - 1) / sg);
       const int64_t per = (items + slots - 1) / slots;  // warps one scheduler runs
       const int64_t waves = (per + n - 1) / n;
-      const double c = std::max(mem, (double)waves * (sg + 2 * K * ry) * std::max(latency, issue * std::min<int64_t>(per, n)));
+      // the share of its time a scheduler's FP64 pipe is busy with nn warps
+      const int nn = (int)std::min<int64_t>(per, n);
+      const double busy = G.dtype == DCP_F64 ? (nn == 1 ? 0.7 : 0.85) : 1.0;
+      const double c = std::max(mem, (double)waves * (sg + 2 * K * ry) * std::max(latency, issue * nn / busy));
       if (c < best * 0.999) best = c, seg = sg, nw = n;
     }
     return best;
@@ -587,7 +646,7 @@ struct Planner {
     double epi = 0;
     for (const StepDesc& st : G.steps)
       for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
-    const double issue = (f64 ? K * 2.0 * 64 * std::max(2, pts - 1) + 60 : K * (11.0 + 4.0 * pts) + 100) +
+    const double issue = (f64 ? (K * 2.0 * 64 * step_ops64(G) + 60) / 0.9 : K * (11.0 + 4.0 * pts) + 100) +
                          K * epi / (double)G.steps.size();
     const double latency = f64 ? 300.0 + 500.0 * K : 130.0 + 45.0 * K;
     double rows = 0, bytes = 0;
@@ -623,7 +682,7 @@ struct Planner {
     epi /= (double)G.steps.size();
     for (int s = 0; s < K; ++s) {
       const double cells = (double)(ty + 2 * (K - 1 - s) * G.radius[1]) * (tx + 2 * (K - 1 - s) * G.radius[2]);
-      if (G.dtype == DCP_F64) t += 1200 + per * cells * (std::max(1, pts - 1) + epi / 128) / 2;
+      if (G.dtype == DCP_F64) t += 1200 + per * cells * (std::min(pts, (int)step_ops64(G) + 1) + epi / 128) / 2;
       else t += std::max(1.0, per / 2.0) * (290.0 * pts / 5 + 0.6 * epi) * std::ceil(cells / 256);
     }
     return t;
@@ -632,8 +691,8 @@ struct Planner {
   // 3-D stars without a prologue run as warp-streamed columns where those are
   // faster, unless a tile option asks for the shared-memory planes: binary64
   // one step per launch, binary32 two.  A warp (nw per scheduler) streams seg + 2 K planes, one
-  // plane costing the larger of its latency and the issue (binary32, about 9
-  // instructions per cell and level) or FP64 pipe time (64 cycles per
+  // plane costing the larger of its latency and the issue (binary32, fitted: 870
+  // cycles for two steps of four rows) or FP64 pipe time (64 cycles per
   // operation of the warp) of the scheduler's warps.
   void choose_columns(Group& G) {
     G.variant = 0;
@@ -660,13 +719,15 @@ struct Planner {
     int64_t bseg = 1;
     // the shared-memory planes: whole tiles of 8 x 32 cells, one operation more
     double best = 1e300;
-    if (f64) {
-      const double padded = (double)nz * ((ny + 7) / 8 * 8) * ((nx + 31) / 32 * 32);
-      best = 0.95 * (std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / 304 + 3000) + 6200) * S;
-    }
+    // (binary32: 63 instructions per cell, 3.84e-3 cycles of the whole GPU)
+    const double padded = (double)nz * ((ny + 7) / 8 * 8) * ((nx + 31) / 32 * 32);
+    best = 0.95 * S *
+           ((f64 ? std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / 304 + 3000)
+                 : std::max(mem, 3.84e-3 * padded * (0.6 + 0.4 * pts / 7 + epi / 252) + 5000)) + 6200);
     const int lx0 = G.lx, cy0 = G.cy;
-    bool column = !f64;
-    for (int K = 1; K <= kmax; ++K)
+    const bool odd = nx % 4 != 0;
+    bool column = false;
+    const int K = kmax;  // (binary32: two steps beat one at every size measured)
       for (int lx : {32, 16})
         for (int cy : {8, 4, 2}) {
           if (!f64 && (cy == 8 || lx != 32)) continue;
@@ -677,8 +738,8 @@ struct Planner {
           const int64_t blocks = (ny + rows_w - 1) / rows_w;
           const double rows = K == 1 ? cy : 2 * cy + 2;  // rows summed per plane, all levels
           const double issue = f64 ? cy * (2 * 64 * (pts - 3 + (cy + 1.0) / cy) + epi) + 100
-                                   : rows * (4.0 * pts + 10 + epi) + (cy + 2 * K) * 9 + 60;
-          const double latency = f64 ? 1500 : 500.0 * K + 300;
+                                   : rows * (52 + 4.0 * pts + epi) + 70 + (odd ? (cy + 2 * K) * 25 : 0);
+          const double latency = f64 ? 1500 : 900 + 700.0 * K;
           const double ends = f64 ? 0.5 : 2.0 * K;  // planes an item pays for beside its own
           // warps per scheduler: what the registers of the form allow without
           // spills (512^3 binary64, 8 rows per lane: 1.22 ms per step at 2,
@@ -810,9 +871,12 @@ struct Planner {
     }
     G.variant = var;
     if (var == 1) {
-      // one warp per CTA: work items end at different times, and a CTA's
-      // slots free together (batch of 4096 instances 2.28 -> 2.13 ms)
-      G.threads = (int)opt(DCP_OPT_STREAM_THREADS, 32);
+      // One warp per CTA: work items end at different times, and a CTA's slots
+      // free together (batch of 4096 instances 2.28 -> 2.13 ms, 4000 x 4100
+      // binary32 16 steps 100 -> 91 us).  Binary64 arrays take two: the few
+      // warps an FP64-bound scheduler needs are then spread over all four
+      // schedulers (5195 x 5862 plain steps 5.15 -> 4.66 ms).
+      G.threads = (int)opt(DCP_OPT_STREAM_THREADS, default_stream_threads(G));
       G.prefetch = (int)opt(DCP_OPT_STREAM_PREFETCH, 1);
       // registers for the four warps per scheduler the plan counts on
       G.min_ctas = (int)opt(DCP_OPT_STREAM_MIN_CTAS, nw >= 4 ? std::min(32, 512 / G.threads) : 0);

@@ -11,7 +11,7 @@
 // once (plus the strip overlap) and written once per DCP_NSTEPS steps.
 //
 // Input rows reach the warp through a ring of DCP_R rows in shared memory that
-// belongs to it alone, filled by asynchronous copies DCP_R - 1 rows ahead: no
+// belongs to it alone, filled by asynchronous copies DCP_R - 2 rows ahead: no
 // block barrier, no register and no scoreboard is held by a load in flight.
 // (Rows prefetched into registers instead left each row waiting for about one
 // memory latency, 0.75 us whatever the number of levels: a warp has six
@@ -71,9 +71,9 @@ static_assert(W > 0 && W % C == 0 && HX + W + K * DCP_RX <= SPAN,
 constexpr int RING = DCP_BC == DCP_BC_FIXED_RING ? RY : 0;  // ring rows
 
 constexpr int R = DCP_R;                           // rows of a warp's ring
-constexpr int D = R - 1;                           // rows requested ahead
+constexpr int D = R - 2;                           // rows requested ahead (rows go in pairs)
 constexpr int ROWB = SPAN * (int)sizeof(T);        // bytes of a row
-static_assert(R >= 2, "the ring holds the current row and at least one ahead");
+static_assert(R >= 4, "the ring holds a pair of rows, the pair before and one ahead");
 
 typedef DcpStParamsT<T> DcpStParams;
 
@@ -242,13 +242,10 @@ __device__ __forceinline__ void dcp_request_checked(unsigned so, int j, const Dc
 constexpr unsigned RMASK = R * ROWB - 1;  // ring offsets wrap by a mask
 static_assert((R & (R - 1)) == 0, "power-of-two ring");
 
-// Input row j from ring row `so` through every level; `a` ends as row
-// j - K*RY after the last.
-template <bool CHECK, bool ROWS, class Pro>
-__device__ __forceinline__ void dcp_row(T (&a)[C], T (&st)[K][NST][C], unsigned so, int j,
-                                        const DcpItem& it, const DcpCols& cols,
-                                        const T (&km)[DCP_NK], Pro& pro, DcpGuard& guard) {
-  union { uint4 v; T t[C]; } x[DCP_NIN];
+union DcpRaw { uint4 v; T t[C]; };
+
+// The lane's vector of ring row `so`, per input.
+__device__ __forceinline__ void dcp_load(DcpRaw (&x)[DCP_NIN], unsigned so, const DcpCols& cols) {
   if (DCP_NLOAD == 0) x[0].v = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
   for (int l = 0; l < DCP_NLOAD; ++l)
@@ -256,6 +253,14 @@ __device__ __forceinline__ void dcp_row(T (&a)[C], T (&st)[K][NST][C], unsigned 
                  : "=r"(x[l].v.x), "=r"(x[l].v.y), "=r"(x[l].v.z), "=r"(x[l].v.w)
                  : "r"(cols.dst + l * (R * ROWB) + so)
                  : "memory");
+}
+
+// Input row j (its loaded vectors x) through every level; `a` ends as row
+// j - K*RY after the last.
+template <bool CHECK, bool ROWS, class Pro>
+__device__ __forceinline__ void dcp_row(T (&a)[C], T (&st)[K][NST][C], const DcpRaw (&x)[DCP_NIN], int j,
+                                        const DcpItem& it, const DcpCols& cols,
+                                        const T (&km)[DCP_NK], Pro& pro, DcpGuard& guard) {
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     T ld[DCP_NIN];
@@ -317,7 +322,8 @@ __device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Pro& pro, Out
   for (int r = 0; r < D; ++r) dcp_request_checked<CHECK>(r * ROWB, j + r, it, cols);
   // Rows [f0, f1] run without row tests: every row such an iteration touches
   // -- level rows from j - K*RY, the requested row j + D -- lies inside the
-  // array and outside a fixed ring (periodic: the requested row).
+  // array and outside a fixed ring (periodic: the requested row).  They go in
+  // pairs (j, j + 1), j < f1.
   const int f0 = DCP_BC == DCP_BC_PERIODIC ? -D : K * RY + RING;
   const int f1 = min(jend - 1, it.ny - (DCP_BC == DCP_BC_PERIODIC ? 0 : RING) - 1 - D);
   T a[C];
@@ -328,26 +334,36 @@ __device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Pro& pro, Out
       long long gi = (long long)(j - K * RY) * it.nx + col0;  // the lane's first element of the finished row
 #pragma unroll 1
       do {
+        // two rows per wait: their levels interleave, and the partial sums
+        // alternate registers
+        dcp_wait_copies<D - 2>();  // this lane's copies of rows j and j + 1 have landed
+        __syncwarp();              // every lane's have, and the pair before has been read
+        DcpRaw x0[DCP_NIN], x1[DCP_NIN];
+        dcp_load(x0, so, cols);
+        dcp_load(x1, (so + ROWB) & RMASK, cols);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {  // pairs: the partial sums alternate registers
-          dcp_wait_copies<D - 1>();  // this lane's copies of row j have landed
-          __syncwarp();              // every lane's have, and row j - 1 has been read
-          dcp_request<CHECK>((so - ROWB) & RMASK, src, cols.in, it, cols);
+        for (int h = 2; h >= 1; --h) {
+          dcp_request<CHECK>((so - h * ROWB) & RMASK, src, cols.in, it, cols);
 #pragma unroll
           for (int l = 0; l < DCP_NLOAD; ++l) src[l] += it.nx;
-          dcp_row<CHECK, true>(a, st, so, j, it, cols, km, pro, guard);
-          so = (so + ROWB) & RMASK;
-          if (j >= jout) output(gi, a);
-          gi += it.nx;
-          ++j;
         }
+        so = (so + 2 * ROWB) & RMASK;
+        dcp_row<CHECK, true>(a, st, x0, j, it, cols, km, pro, guard);
+        if (j >= jout) output(gi, a);
+        gi += it.nx;
+        dcp_row<CHECK, true>(a, st, x1, j + 1, it, cols, km, pro, guard);
+        if (j + 1 >= jout) output(gi, a);
+        gi += it.nx;
+        j += 2;
       } while (j < f1);
     }
     if (j < jend) {
       dcp_wait_copies<D - 1>();
       __syncwarp();
-      dcp_request_checked<CHECK>((so - ROWB) & RMASK, j + D, it, cols);
-      dcp_row<CHECK, false>(a, st, so, j, it, cols, km, pro, guard);
+      DcpRaw x[DCP_NIN];
+      dcp_load(x, so, cols);
+      dcp_request_checked<CHECK>((so - 2 * ROWB) & RMASK, j + D, it, cols);
+      dcp_row<CHECK, false>(a, st, x, j, it, cols, km, pro, guard);
       so = (so + ROWB) & RMASK;
       if (j >= jout) output((long long)(j - K * RY) * it.nx + col0, a);
       ++j;

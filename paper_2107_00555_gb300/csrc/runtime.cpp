@@ -970,7 +970,7 @@ void apply_config(GraphImpl& g, int gi, const TuneCfg& cfg) {
   G.cx = cfg[4] == 2 && G.tile[2] % 2 == 0 && G.radius[2] <= 2 ? 2 : 1;
   if (G.variant == 1) {
     auto th = g.options.find(DCP_OPT_STREAM_THREADS);
-    G.threads = th == g.options.end() ? 32 : (int)th->second;
+    G.threads = th == g.options.end() ? default_stream_threads(G) : (int)th->second;
     G.prefetch = cfg[3] > 0 ? cfg[3] : 1;
     G.min_ctas = cfg[4] > 1 ? cfg[4] : 0;
     if (G.kind == GroupKind::Batch) {
