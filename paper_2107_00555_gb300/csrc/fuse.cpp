@@ -746,7 +746,7 @@ struct Planner {
           // 1.41 at 3; 300 x 333 x 381 binary32: 59 us at 3, 72 at 4)
           const int nmax = f64 && cy == 8 ? 2 : 3;
           for (int n = 1; n <= nmax; ++n)
-            for (int wv = 1; wv <= 16; ++wv) {  // items in whole waves of n warps per scheduler
+            for (int wv = 1; wv <= (n == nmax ? 16 : 1); ++wv) {  // whole waves of the resident warps
               const int64_t segs = (int64_t)wv * n * 608 / (strips * blocks);
               if (segs < 1) continue;
               const int64_t sg = (nz + std::min(segs, nz) - 1) / std::min(segs, nz);
@@ -807,15 +807,16 @@ struct Planner {
     int64_t seg = 0;
     int nw = 4;
     if (G.kind == GroupKind::Stencil && var == 1 && cells > 0) {
-      double best = stream_cycles(G, G.depth, seg, nw) + launch;
-      best *= (S + G.depth - 1) / G.depth;
+      // (the last launch of an uneven split runs fewer steps)
+      auto total = [&](double cycles, int K) { return cycles * S / K + launch * ((S + K - 1) / K); };
+      double best = total(stream_cycles(G, G.depth, seg, nw), G.depth);
       if (free_depth)
         for (int most = 1; most <= std::min(S, G.dtype == DCP_F32 ? 10 : 4); ++most) {
           const int K = even(most);
           int64_t sg;
           int n;
           if (!stream_eligible(G, K)) continue;
-          const double c = (stream_cycles(G, K, sg, n) + launch) * ((S + K - 1) / K);
+          const double c = total(stream_cycles(G, K, sg, n), K);
           if (c < best) best = c, G.depth = K, seg = sg, nw = n;
         }
       // Small grids run faster in shared-memory tiles, where every cell of a
@@ -829,7 +830,7 @@ struct Planner {
             for (int ty : {4, 8, 12, 14, 16, 24, 32}) {
               const long smem = 2L * (ty + 2 * K * G.radius[1]) * (tx + 2 * K * G.radius[2]) * dtype_size(G.dtype);
               if (smem > 96 * 1024) continue;
-              const double c = (tile_cycles(G, K, ty, tx) + 1.3 * launch) * ((S + K - 1) / K);
+              const double c = total(tile_cycles(G, K, ty, tx), K) + 0.3 * launch * ((S + K - 1) / K);
               if (c < best) {
                 best = c;
                 var = 0;
@@ -850,7 +851,7 @@ struct Planner {
         const int K = free_depth ? even(most) : G.depth;
         if (!stream_eligible(G, K)) continue;
         for (int sg : {16, 32, 64, 128, 256}) {
-          const double c = (batch_cycles(G, K, sg) + launch) * ((S + K - 1) / K);
+          const double c = batch_cycles(G, K, sg) * S / K + launch * ((S + K - 1) / K);
           if (c < best) best = c, G.depth = K, seg = sg;
         }
       }
