@@ -137,11 +137,15 @@ def _check(name, status):
         raise DcpError(status, name, load().dcp_last_error().decode(errors="replace"))
 
 
+_ARR = {}  # length -> void*[length]
+
+
 def _ptrs(seq):
-    arr = (_P * max(1, len(seq)))()
-    for i, p in enumerate(seq):
-        arr[i] = p
-    return arr
+    n = max(1, len(seq))
+    t = _ARR.get(n)
+    if t is None:
+        t = _ARR[n] = _P * n
+    return t(*seq)
 
 
 def dcp_graph_create():

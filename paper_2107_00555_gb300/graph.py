@@ -33,6 +33,16 @@ def _numpy_dtype(code):
             C.DCP_I32: np.int32, C.DCP_I64: np.int64}[code]
 
 
+def _raw_stream(stream):
+    """cudaStream_t of a torch stream, by default torch's current one.  The
+    default skips building a Stream object (measured: 6 of the 27 us of a small
+    program's call)."""
+    import torch
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
 class Graph:
     """A dcp program.  Values are integer handles returned by the builder calls."""
 
@@ -44,6 +54,7 @@ class Graph:
         self.dtype = {}
         self.fused = False
         self.n_kernels = None
+        self._specs = {}  # value -> (torch shape, torch dtype), filled on first use
 
     # -- construction --------------------------------------------------------
     def input(self, dtype, shape):
@@ -105,6 +116,22 @@ class Graph:
         return json.loads(C.dcp_plan_info(self._h))
 
     # -- execution -------------------------------------------------------------
+    def _spec(self, v):
+        import torch
+        s = self._specs.get(v)
+        if s is None:
+            s = self._specs[v] = (torch.Size(self.shape[v]), _torch_dtype(self.dtype[v]))
+        return s
+
+    def _check_tensors(self, ts, vs, what):
+        """Every tensor against its value; _check_tensor names what is wrong."""
+        import torch
+        for i, (t, v) in enumerate(zip(ts, vs)):
+            shape, dtype = self._spec(v)
+            if not (isinstance(t, torch.Tensor) and t.is_cuda and t.shape == shape
+                    and t.dtype is dtype and t.is_contiguous()):
+                self._check_tensor(t, v, "%s %d" % (what, i))
+
     def _check_tensor(self, t, v, what):
         import torch
         if not isinstance(t, torch.Tensor):
@@ -120,24 +147,21 @@ class Graph:
 
     def empty_outputs(self, device=None):
         import torch
-        return [torch.empty(self.shape[v], dtype=_torch_dtype(self.dtype[v]),
-                            device=device or "cuda") for v in self.outputs]
+        device = device or "cuda"
+        specs = [self._spec(v) for v in self.outputs]
+        return [torch.empty(shape, dtype=dtype, device=device) for shape, dtype in specs]
 
     def run(self, inputs, outputs=None, stream=None):
         """Run on CUDA tensors (asynchronous on ``stream``, default: torch's current)."""
-        import torch
         if len(inputs) != len(self.inputs):
             raise ValueError("expected %d inputs" % len(self.inputs))
-        for i, (t, v) in enumerate(zip(inputs, self.inputs)):
-            self._check_tensor(t, v, "input %d" % i)
+        self._check_tensors(inputs, self.inputs, "input")
         if outputs is None:
             outputs = self.empty_outputs(inputs[0].device if inputs else None)
-        for j, (t, v) in enumerate(zip(outputs, self.outputs)):
-            self._check_tensor(t, v, "output %d" % j)
-        if stream is None:
-            stream = torch.cuda.current_stream()
+        else:
+            self._check_tensors(outputs, self.outputs, "output")
         C.dcp_run(self._h, [t.data_ptr() for t in inputs], [t.data_ptr() for t in outputs],
-                  stream.cuda_stream)
+                  _raw_stream(stream))
         return outputs
 
     def prepare(self, inputs, outputs=None):
@@ -161,8 +185,7 @@ class Graph:
         keep = (list(inputs), list(outputs))
 
         def run(stream=None):
-            s = (stream or torch.cuda.current_stream()).cuda_stream
-            C._check("dcp_run", lib.dcp_run(h, ins, outs, s))
+            C._check("dcp_run", lib.dcp_run(h, ins, outs, _raw_stream(stream)))
             return keep[1]
 
         run.outputs = outputs
@@ -224,19 +247,15 @@ class Graph:
     def adjoint(self, inputs, out_grads, in_grads=None, tape_budget_bytes=1 << 62, stream=None):
         """Reverse pass: cotangents of the inputs given those of the outputs."""
         import torch
-        for i, (t, v) in enumerate(zip(inputs, self.inputs)):
-            self._check_tensor(t, v, "input %d" % i)
-        for j, (t, v) in enumerate(zip(out_grads, self.outputs)):
-            self._check_tensor(t, v, "output cotangent %d" % j)
+        self._check_tensors(inputs, self.inputs, "input")
+        self._check_tensors(out_grads, self.outputs, "output cotangent")
         if in_grads is None:
             in_grads = [torch.empty_like(t) for t in inputs]
-        for i, (t, v) in enumerate(zip(in_grads, self.inputs)):
-            self._check_tensor(t, v, "input cotangent %d" % i)
-        if stream is None:
-            stream = torch.cuda.current_stream()
+        else:
+            self._check_tensors(in_grads, self.inputs, "input cotangent")
         C.dcp_run_adjoint(self._h, [t.data_ptr() for t in inputs],
                           [t.data_ptr() for t in out_grads], [t.data_ptr() for t in in_grads],
-                          tape_budget_bytes, stream.cuda_stream)
+                          tape_budget_bytes, _raw_stream(stream))
         return in_grads
 
     def prepare_adjoint(self, tape_budget_bytes=1 << 62):
