@@ -453,7 +453,8 @@ class Stencil(Workload):
         # terms per cell (a multiply and an add each, except the first add:
         # 2p - 1 flops; 13 for the 7-point step).  Alongside: the FP64
         # instructions the kernels execute per useful cell and step (p - 1
-        # on a deferred common weight, plus one multiply at chunk ends; p for
+        # on a deferred common weight, plus one multiply at chunk ends; fewer
+        # where a kernel form shares the star's pair sums between cells; p for
         # the plain weighted sum), and the compulsory device-memory traffic
         # of one launch (the grid read once and written once).
         # (a sharded rank's launches process its slab with halos)
@@ -467,8 +468,17 @@ class Stencil(Workload):
 
     def plan_model(self, plan):
         """FP64 instructions per useful cell and step, averaged over the run,
-        from the plan's per-step deferral factors."""
+        from the plan's per-step deferral factors and the kernel form: columns
+        of r rows per lane take (r + 1) / r pair sums for two pairs of a
+        7-point star, the warp stream one for both pairs of a 5-point star."""
         total, steps = 0.0, 0
+        grp = plan["groups"][0]
+        deferred = self.npts - 1
+        if grp.get("kernel_form") == "column":
+            r = grp["rows_per_lane"]
+            deferred = self.npts - 3 + (r + 1) / r
+        elif grp.get("kernel_form") == "stream" and self.npts == 5:
+            deferred = self.npts - 2
         for l in plan["launches"]:
             lo, hi = l["steps"]
             scales = l.get("deferred_scales")
@@ -477,7 +487,7 @@ class Stencil(Workload):
                     total += self.npts          # one multiply + p - 1 FMAs
                 else:
                     f = scales[k] if k < len(scales) else 1
-                    total += (self.npts - 1) + (0 if f == 1 else 1)
+                    total += deferred + (0 if f == 1 else 1)
                 steps += 1
         self.fp64_inst_per_cell_step = total / max(1, steps)
 
