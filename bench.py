@@ -466,29 +466,32 @@ class Stencil(Workload):
                 "fp64_inst_per_cell_step": self.fp64_inst_per_cell_step,
                 "hbm_bytes": 2 * cells * self.size}
 
-    def plan_model(self, plan):
-        """FP64 instructions per useful cell and step, averaged over the run,
-        from the plan's per-step deferral factors and the kernel form: columns
-        of r rows per lane take (r + 1) / r pair sums for two pairs of a
-        7-point star, the warp stream one for both pairs of a 5-point star."""
+    def plan_model(self, *plans):
+        """FP64 instructions per useful cell and step, averaged over the runs
+        of the plans (a sharded rank runs one graph per chunk of steps, each
+        with a kernel form of its own), from the per-step deferral factors and
+        the kernel form: columns of r rows per lane take (r + 1) / r pair sums
+        for two pairs of a 7-point star, the warp stream one for both pairs of
+        a 5-point star."""
         total, steps = 0.0, 0
-        grp = plan["groups"][0]
-        deferred = self.npts - 1
-        if grp.get("kernel_form") == "column":
-            r = grp["rows_per_lane"]
-            deferred = self.npts - 3 + (r + 1) / r
-        elif grp.get("kernel_form") == "stream" and self.npts == 5:
-            deferred = self.npts - 2
-        for l in plan["launches"]:
-            lo, hi = l["steps"]
-            scales = l.get("deferred_scales")
-            for k in range(hi - lo):
-                if scales is None:
-                    total += self.npts          # one multiply + p - 1 FMAs
-                else:
-                    f = scales[k] if k < len(scales) else 1
-                    total += deferred + (0 if f == 1 else 1)
-                steps += 1
+        for plan in plans:
+            for l in plan["launches"]:
+                grp = plan["groups"][l["group"]]
+                deferred = self.npts - 1
+                if grp.get("kernel_form") == "column":
+                    r = grp["rows_per_lane"]
+                    deferred = self.npts - 3 + (r + 1) / r
+                elif grp.get("kernel_form") == "stream" and self.npts == 5:
+                    deferred = self.npts - 2
+                lo, hi = l["steps"]
+                scales = l.get("deferred_scales")
+                for k in range(hi - lo):
+                    if scales is None:
+                        total += self.npts          # one multiply + p - 1 FMAs
+                    else:
+                        f = scales[k] if k < len(scales) else 1
+                        total += deferred + (0 if f == 1 else 1)
+                    steps += 1
         self.fp64_inst_per_cell_step = total / max(1, steps)
 
     def describe(self):
@@ -640,8 +643,7 @@ class Stencil(Workload):
         plan0 = g0.plan()
         self.kernels = [l["kernel"] for l in plan0["launches"]]
         self.n_launch = sum(len(self.local_graphs[c.steps].plan()["launches"]) for c in plan.chunks)
-        self.plan_model({"launches": [l for c in plan.chunks
-                                      for l in self.local_graphs[c.steps].plan()["launches"]]})
+        self.plan_model(*[self.local_graphs[c.steps].plan() for c in plan.chunks])
         self.roof_cells = 1
         for d in plan.local_shape:
             self.roof_cells *= d
