@@ -217,8 +217,9 @@ std::string red_op_fn(const GraphImpl& g, const std::vector<int>& reds) {
 }
 
 // A kernel's name hashes its generated prefix together with the
-// hand-written skeletons it includes, so the name (and the compiled-module
-// caches keyed by the source) changes exactly when one of them changes.
+// hand-written skeletons it includes (and those they include), so the name
+// (and the compiled-module caches keyed by the source) changes exactly when
+// one of them changes.
 uint64_t skeleton_hash(const std::string& body) {
   const std::pair<const char*, const char*> skel[] = {
       {"k_map.cuh", kernel_map_source()},
@@ -230,19 +231,28 @@ uint64_t skeleton_hash(const std::string& body) {
       {"k_stencil_adj.cuh", kernel_adj_source()},
       {"k_stencil2d_coop.cuh", kernel_coop_source()},
       {"k_tanh64.cuh", kernel_tanh64_source()},
+      {"k_tanh64_table.cuh", kernel_tanh64_table_source()},
       {"k_stencil3d_col.cuh", kernel_column_source()}};
-  unsigned used = 0;
-  for (size_t i = 0; i < sizeof skel / sizeof skel[0]; ++i)
-    if (body.find(std::string("#include \"") + skel[i].first + "\"") != std::string::npos) used |= 1u << i;
+  constexpr size_t N = sizeof skel / sizeof skel[0];
+  auto included = [&](const std::string& by) {
+    unsigned m = 0;
+    for (size_t i = 0; i < N; ++i)
+      if (by.find(std::string("#include \"") + skel[i].first + "\"") != std::string::npos) m |= 1u << i;
+    return m;
+  };
+  const unsigned used = included(body);
   // (the skeletons never change within a process: one hash per set of them)
   static std::mutex mu;
   static std::map<unsigned, uint64_t> known;
   std::lock_guard<std::mutex> lk(mu);
   auto it = known.find(used);
   if (it != known.end()) return it->second;
+  unsigned all = used;  // with the skeletons they include themselves
+  for (size_t i = 0; i < N; ++i)
+    if (used >> i & 1u) all |= included(skel[i].second);
   std::string text = device_header_source();
-  for (size_t i = 0; i < sizeof skel / sizeof skel[0]; ++i)
-    if (used >> i & 1u) text += skel[i].second;
+  for (size_t i = 0; i < N; ++i)
+    if (all >> i & 1u) text += skel[i].second;
   return known[used] = fnv1a(text);
 }
 
