@@ -1270,8 +1270,6 @@ std::string describe_plan(const GraphImpl& g) {
          << ", \"min_ctas\": " << G.min_ctas;
     if (G.kind == GroupKind::Stencil && G.variant == 3)
       os << ", \"rows_per_lane\": " << G.cy << ", \"lanes_x\": " << G.lx;
-    if (G.kind == GroupKind::Stencil && G.variant == 3)
-      os << ", \"rows_per_lane\": " << G.cy << ", \"lanes_x\": " << G.lx;
     int epi = 0;
     for (const StepDesc& s : G.steps) epi += (int)s.epi.size();
     if (G.kind == GroupKind::AdjTile)
