@@ -115,22 +115,44 @@ struct Planner {
     finalize();
   }
 
-  // Maps reached from value m that may join the prologue of reductions along
-  // `axis` of the group that will replace map group gi: same space, read only
-  // by such maps or by reductions along that axis, every operand computed
-  // there or before.  Collects them in `maps` and the reductions in nred.
-  bool axis_closure(int m, const Group& M, int gi, int axis, std::set<int>& maps, std::set<int>& reds) const {
-    for (int u : users[m]) {
-      if (!live[u] || in_vec(M.members, u) || maps.count(u)) continue;
-      const Node& un = g.nodes[u];
-      if (un.kind == Kind::Reduce && un.axis == axis) {
-        reds.insert(u);
-        continue;
+  // What an axis-reduce group will hold once the rest of its prologue has
+  // been planned: room other reductions over the same space must leave.
+  struct AxisDue {
+    std::set<int> maps, reds, loads, scalars;
+  };
+  std::map<int, AxisDue> axis_due;
+
+  // The maps reached from those of map group M (group gi) that may join the
+  // prologue of reductions along `axis` of the group that will replace it:
+  // same space, read only by such maps or by reductions along that axis,
+  // every operand computed there or before.
+  bool axis_closure(const Group& M, int gi, int axis, AxisDue& due) const {
+    const std::set<int> own(M.members.begin(), M.members.end());
+    std::vector<int> todo = M.members;
+    while (!todo.empty()) {
+      const int m = todo.back();
+      todo.pop_back();
+      if (is_out[m] || g.nodes[m].kind != Kind::Map) return false;
+      for (int u : users[m]) {
+        if (!live[u] || own.count(u) || due.maps.count(u)) continue;
+        const Node& un = g.nodes[u];
+        if (un.kind == Kind::Reduce && un.axis == axis) {
+          due.reds.insert(u);
+          continue;
+        }
+        if (un.kind != Kind::Map || un.shape != M.shape) return false;
+        due.maps.insert(u);
+        todo.push_back(u);
       }
-      if (un.kind != Kind::Map || un.shape != M.shape || is_out[u]) return false;
-      maps.insert(u);
-      if (!axis_closure(u, M, gi, axis, maps, reds)) return false;
     }
+    due.loads.insert(M.loads.begin(), M.loads.end());
+    due.scalars.insert(M.scalars.begin(), M.scalars.end());
+    for (int u : due.maps)
+      for (int b : g.nodes[u].in) {
+        if (own.count(b) || due.maps.count(b)) continue;
+        if (g.nodes[b].kind != Kind::Input && !(g.value_group[b] >= 0 && g.value_group[b] < gi)) return false;
+        (g.nodes[b].shape.empty() ? due.scalars : due.loads).insert(b);
+      }
     return true;
   }
 
@@ -236,7 +258,7 @@ struct Planner {
     if (fsub() && !g.groups.empty()) {
       int li = (int)g.groups.size() - 1;
       Group& G = g.groups[li];
-      if (same_space(G) && (int)G.reds.size() < kMaxIO && available_before(a, li)) {
+      if (same_space(G) && available_before(a, li) && axis_room(G, li, a)) {
         G.reds.push_back(v);
         g.value_group[v] = li;
         add_operand(G, li, a);
@@ -249,35 +271,20 @@ struct Planner {
     R.shape = an.shape;
     R.axis = n.axis;
     bool absorbed = false;
-    std::set<int> later;
+    AxisDue due;
     if (fsub() && gi >= 0 && gi == (int)g.groups.size() - 1 &&
         g.groups[gi].kind == GroupKind::Map && computed_in(gi, a)) {
       const Group& M = g.groups[gi];
-      bool ok = M.reds.empty() && M.shape == an.shape;
-      std::set<int> reds;
-      for (int m : M.members) {
-        if (is_out[m] || g.nodes[m].kind != Kind::Map) ok = false;
-        ok = ok && axis_closure(m, M, gi, n.axis, later, reds);
-      }
-      // the operands of the maps still to come, and the limits of one kernel
-      std::set<int> loads(M.loads.begin(), M.loads.end()), scalars(M.scalars.begin(), M.scalars.end());
-      for (int u : later)
-        for (int b : g.nodes[u].in) {
-          if (in_vec(M.members, b) || later.count(b)) continue;
-          const bool known = g.nodes[b].kind == Kind::Input || (g.value_group[b] >= 0 && g.value_group[b] < gi);
-          ok = ok && known;
-          (g.nodes[b].shape.empty() ? scalars : loads).insert(b);
-        }
-      const int nred = (int)reds.size();
+      bool ok = M.reds.empty() && M.shape == an.shape && axis_closure(M, gi, n.axis, due);
       // binary64 maps with exp, sin and the like are bound by the FP64 pipe,
       // which the map kernel keeps busier than a row tree: maps still to come
       // then stay in its one pass (8063 x 140 binary64 columns 99 us against
       // 168 in one kernel, 6751 x 1810 rows 784 against 848)
       double cost = 0;
       for (int m : M.members) cost += op_cycles(g.nodes[m].op, an.dtype);
-      if (an.dtype == DCP_F64 && !later.empty() && cost > 12 * op_cycles(DCP_ADD, DCP_F64)) ok = false;
-      if ((int)loads.size() > kMaxIO || (int)scalars.size() > kMaxIO) ok = false;
-      if (ok && nred <= kMaxIO) {
+      if (an.dtype == DCP_F64 && !due.maps.empty() && cost > 12 * op_cycles(DCP_ADD, DCP_F64)) ok = false;
+      if (ok && (int)due.loads.size() <= kMaxIO && (int)due.scalars.size() <= kMaxIO &&
+          (int)due.reds.size() <= kMaxIO) {
         R.members = M.members;
         R.loads = M.loads;
         R.scalars = M.scalars;
@@ -291,8 +298,23 @@ struct Planner {
     int ri = (int)g.groups.size() - 1;
     g.value_group[v] = ri;
     for (int m : R.members) g.value_group[m] = ri;
-    if (absorbed)
-      for (int u : later) axis_map[u] = ri;
+    if (absorbed) {
+      for (int u : due.maps) axis_map[u] = ri;
+      axis_due[ri] = due;
+    }
+  }
+
+  // Can axis-reduce group gi take another reduction, of value a, beside those
+  // its own prologue still brings?
+  bool axis_room(const Group& G, int gi, int a) const {
+    std::set<int> reds(G.reds.begin(), G.reds.end()), loads(G.loads.begin(), G.loads.end());
+    auto due = axis_due.find(gi);
+    if (due != axis_due.end()) {
+      reds.insert(due->second.reds.begin(), due->second.reds.end());
+      loads.insert(due->second.loads.begin(), due->second.loads.end());
+    }
+    if (!computed_in(gi, a)) loads.insert(a);
+    return (int)reds.size() < kMaxIO && (int)loads.size() <= kMaxIO;
   }
 
   void plan_reduce(int v) {

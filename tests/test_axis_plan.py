@@ -1,0 +1,49 @@
+"""Maps fused into the prologue of axis reductions: what the planner takes in,
+and what it leaves room for."""
+import pytest
+
+from paper_2107_00555_gb300 import Graph
+from paper_2107_00555_gb300 import _capi as C
+
+SHAPE = (30, 41)
+
+
+def _groups(g, flags=C.DCP_FUSE_ALL):
+    g.fuse(flags)
+    return [(p["kind"], p["members"], p["loads"], p["reductions"]) for p in g.plan()["groups"]]
+
+
+def test_other_reductions_leave_room_for_those_of_the_prologue():
+    """A reduction of the prologue's later maps always finds a place in its
+    kernel (16 reductions), whatever was reduced in between."""
+    g = Graph()
+    x = g.input("f32", SHAPE)
+    others = [g.input("f32", SHAPE) for _ in range(5)]
+    y = g.map("square", [x])
+    g.output(g.reduce(y, "sum", axis=1))
+    for o in others:
+        for op in ("sum", "min", "max"):
+            g.output(g.reduce(o, op, axis=1))
+    z = g.map("abs", [y])
+    for op in ("sum", "min", "max"):
+        g.output(g.reduce(z, op, axis=1))
+    kinds = _groups(g)
+    assert kinds[0] == ("axis_reduce", 2, 5, 16)  # y, z; 4 + 12 reductions of 1 + 4 arrays
+    assert kinds[1:] == [("axis_reduce", 0, 1, 3)]
+
+
+def test_other_reductions_leave_room_for_the_loads_of_the_prologue():
+    """16 loads per kernel: the maps still to come read 13 arrays."""
+    g = Graph()
+    x = g.input("f32", SHAPE)
+    operands = [g.input("f32", SHAPE) for _ in range(12)]
+    others = [g.input("f32", SHAPE) for _ in range(5)]
+    y = g.map("square", [x])
+    g.output(g.reduce(y, "sum", axis=0))
+    for o in others:
+        g.output(g.reduce(o, "sum", axis=0))
+    z = y
+    for o in operands:
+        z = g.map("add", [z, o])
+    g.output(g.reduce(z, "sum", axis=0))
+    assert _groups(g) == [("axis_reduce", 13, 16, 5), ("axis_reduce", 0, 2, 2)]
