@@ -282,6 +282,7 @@ struct Planner {
       // 168 in one kernel, 6751 x 1810 rows 784 against 848)
       double cost = 0;
       for (int m : M.members) cost += op_cycles(g.nodes[m].op, an.dtype);
+      if (!due.maps.empty() && !fmaps()) ok = false;  // (maps are not to be fused with one another)
       if (an.dtype == DCP_F64 && !due.maps.empty() && cost > 12 * op_cycles(DCP_ADD, DCP_F64)) ok = false;
       if (ok && (int)due.loads.size() <= kMaxIO && (int)due.scalars.size() <= kMaxIO &&
           (int)due.reds.size() <= kMaxIO) {

@@ -47,3 +47,15 @@ def test_other_reductions_leave_room_for_the_loads_of_the_prologue():
         z = g.map("add", [z, o])
     g.output(g.reduce(z, "sum", axis=0))
     assert _groups(g) == [("axis_reduce", 13, 16, 5), ("axis_reduce", 0, 2, 2)]
+
+
+def test_maps_stay_apart_unless_maps_are_to_be_fused():
+    """DCP_FUSE_SUBGRAPH alone takes a map into the reduction that reads it, and
+    fuses no map with another."""
+    g = Graph()
+    x = g.input("f32", SHAPE)
+    y = g.map("square", [x])
+    g.output(g.reduce(y, "sum", axis=1))
+    g.output(g.reduce(g.map("abs", [g.map("sub", [y, x])]), "max", axis=1))
+    kinds = _groups(g, C.DCP_FUSE_SUBGRAPH)
+    assert all(members <= 1 for _, members, _, _ in kinds)
