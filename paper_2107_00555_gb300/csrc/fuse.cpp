@@ -721,8 +721,7 @@ struct Planner {
     G.variant = 0;
     const auto has = [&](int key) { return g.options.count(key) > 0; };
     if (!column_eligible(g, G) || has(DCP_OPT_TILE_X) || has(DCP_OPT_TILE_Y) || has(DCP_OPT_TILE_Z) ||
-        has(DCP_OPT_CELLS_PER_THREAD) || G.shape[0] * G.shape[1] * G.shape[2] == 0 ||
-        G.shape[1] * G.shape[2] > 0x7fffffff)  // (offsets within a plane are 32-bit)
+        has(DCP_OPT_CELLS_PER_THREAD) || G.shape[0] * G.shape[1] * G.shape[2] == 0)
       return;
     const bool f64 = G.dtype == DCP_F64;
     const int S = (int)G.steps.size();

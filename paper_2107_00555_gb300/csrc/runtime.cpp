@@ -819,7 +819,8 @@ namespace {
 // A tuned configuration: depth, tz, ty, tx, and for 3-D stencils the cells
 // per thread along x, for 2-D tile kernels the threads per CTA (32 or more;
 // smaller values mean the default 256) (stream kernels: tz = -1, ty = rows
-// per item, tx = prefetch depth).
+// per item, tx = prefetch depth; 3-D columns: tz = -3, ty = rows per lane,
+// tx = planes per item, then the lanes along x).
 typedef std::array<int, 5> TuneCfg;
 std::mutex g_tune_mu;
 std::map<std::string, TuneCfg> g_tune_cache;  // signature -> configuration
@@ -864,6 +865,9 @@ std::string group_signature(const GraphImpl& g, const Group& G, int device_sms) 
   for (auto o : G.offsets) os << o << ",";
   os << "|p" << G.members.size() << "," << G.post.size() << "," << G.reds.size();
   for (const StepDesc& s : G.steps) os << "," << s.epi.size();
+  // columns suit only some weights and options of one neighbourhood: groups
+  // that may run them and groups that may not are tuned apart
+  if (column_eligible(g, G)) os << "|col";
   char h[32];
   std::snprintf(h, sizeof h, "%016" PRIx64, fnv1a(os.str()));
   return h;
@@ -953,8 +957,19 @@ std::vector<TuneCfg> tune_candidates(const Group& G, int sms) {
   return c;
 }
 
+// Can the group run the configuration?  The column form computes the wrong
+// sums for a group that is not eligible, whatever a cache file holds.
+bool config_ok(const GraphImpl& g, const Group& G, const TuneCfg& cfg) {
+  if (cfg[1] != -3) return true;
+  const int cy = cfg[2], lx = cfg[4], depth = cfg[0];
+  if (!column_eligible(g, G) || cfg[3] < 1 || depth < 1 || depth > (int)G.steps.size()) return false;
+  if (G.dtype == DCP_F64) return depth == 1 && (cy == 2 || cy == 4 || cy == 8) && (lx == 16 || lx == 32);
+  return depth <= 2 && (cy == 2 || cy == 4) && lx == 32;
+}
+
 void apply_config(GraphImpl& g, int gi, const TuneCfg& cfg) {
   Group& G = g.groups[gi];
+  if (!config_ok(g, G, cfg)) fail(DCP_E_UNSUPPORTED, "3-D columns do not suit this stencil group");
   G.depth = cfg[0];
   G.variant = cfg[1] == -1 ? 1 : (cfg[1] == -2 ? 2 : (cfg[1] == -3 ? 3 : 0));
   if (G.variant == 3) {
@@ -1031,7 +1046,7 @@ static void autotune(GraphImpl& g, const std::vector<const void*>& ptr, cudaStre
     }
     std::string key = group_signature(g, G, rt.sms);
     auto hit = g_tune_cache.find(key);
-    if (hit != g_tune_cache.end()) {
+    if (hit != g_tune_cache.end() && config_ok(g, G, hit->second)) {
       apply_config(g, gi, hit->second);
       launch_group(g, gi, ptr, s);
       continue;
