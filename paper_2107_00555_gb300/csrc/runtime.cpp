@@ -1051,9 +1051,10 @@ static void autotune(GraphImpl& g, const std::vector<const void*>& ptr, cudaStre
       launch_group(g, gi, ptr, s);
       continue;
     }
-    TuneCfg best = {G.depth, G.variant == 1 ? -1 : (G.variant == 2 ? -2 : G.tile[0]),
-                    G.variant == 1 ? G.seg : G.tile[1], G.variant == 1 ? G.prefetch : G.tile[2],
-                    G.variant == 2 ? G.threads : G.cx};
+    // the planner's choice, kept when no candidate can be timed
+    TuneCfg best = {G.depth, G.tile[0], G.tile[1], G.tile[2], G.cx};
+    if (G.variant == 1) best = {G.depth, -1, G.seg, G.prefetch, std::max(1, G.min_ctas)};
+    if (G.variant == 3) best = {G.depth, -3, G.cy, G.seg, G.lx};
     float best_ms = 1e30f;
     for (const auto& cfg : tune_candidates(G, rt.sms)) {
       try {
