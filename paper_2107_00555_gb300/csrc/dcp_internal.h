@@ -28,6 +28,17 @@ void set_last_error(const std::string& msg);
 void check_cuda(cudaError_t e, const char* what);
 void check_cu(CUresult r, const char* what);
 
+// Within its scope this thread may load modules and allocate while a stream
+// captures (such calls are no part of the captured work, and the default
+// capture mode refuses them).
+struct CaptureRelaxed {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CaptureRelaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~CaptureRelaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  CaptureRelaxed(const CaptureRelaxed&) = delete;
+  CaptureRelaxed& operator=(const CaptureRelaxed&) = delete;
+};
+
 // Driver API entry points (driver.cpp), resolved through the runtime.
 struct Driver {
   CUresult (*ctxGetCurrent)(CUcontext*) = nullptr;

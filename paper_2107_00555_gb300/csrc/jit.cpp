@@ -135,6 +135,7 @@ CUfunction load_function(const std::string& src, const std::string& name, double
   }
   CubinRef cubin = nvrtc_compile(src, name, ms, nullptr);
   CUmodule mod;
+  const CaptureRelaxed relaxed;  // (a variant may be loaded inside a caller's capture)
   check_cu(drv().moduleLoadData(&mod, cubin->data()), "cuModuleLoadData");
   CUfunction fn;
   check_cu(drv().moduleGetFunction(&fn, mod, name.c_str()), "cuModuleGetFunction");

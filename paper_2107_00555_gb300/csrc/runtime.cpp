@@ -356,6 +356,7 @@ static void* group_partials(GraphImpl& g, int gi, int64_t slots) {
   GroupRT& R = rt.grt[gi];
   if (slots < 1) slots = 1;
   if (!R.partials || R.partial_slots < slots) {
+    const CaptureRelaxed relaxed;  // (a variant with more CTAs may first run inside a caller's capture)
     R.partials = dalloc(rt, (size_t)slots * g.groups[gi].reds.size() * 8);
     R.partial_slots = (int)slots;
   }
@@ -542,6 +543,19 @@ static void* arm_guard(GraphImpl& g, const LaunchSpec& ls, cudaStream_t s) {
 static void launch_coop(GraphImpl& g, LaunchSpec& ls, const StParamsH& sp, int64_t tiles,
                         cudaStream_t s);
 
+// The element-wise variant of a streamed stencil launch, compiled and loaded
+// when a buffer off the vector boundary is first seen (by any thread, possibly
+// inside a caller's capture).
+static void load_scalar_variant(const GraphImpl& g, const Group& G, LaunchSpec& ls) {
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lk(mu);
+  if (ls.fn_scalar) return;
+  ls.code_scalar = gen_stencil_kernel(g, G, ls.s0, ls.s1, 1);
+  CUfunction fn = load_function(ls.code_scalar.source, ls.code_scalar.name, nullptr, nullptr);
+  ls.occ_scalar = prepare_function(fn, ls.code_scalar);
+  ls.fn_scalar = fn;
+}
+
 static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const void*>& ptr,
                            cudaStream_t s) {
   auto& rt = *g.rt;
@@ -582,11 +596,7 @@ static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const
     uintptr_t mis = 0;
     for (int i = 0; i < kMaxIO; ++i) mis |= (uintptr_t)p.ld[i] | (uintptr_t)p.st[i];
     if (mis % (uintptr_t)(ls.code.vec * dtype_size(G.dtype))) {
-      if (!ls.fn_scalar) {
-        ls.code_scalar = gen_stencil_kernel(g, G, ls.s0, ls.s1, 1);
-        ls.fn_scalar = load_function(ls.code_scalar.source, ls.code_scalar.name, nullptr, nullptr);
-        ls.occ_scalar = prepare_function(ls.fn_scalar, ls.code_scalar);
-      }
+      load_scalar_variant(g, G, ls);
       fn = ls.fn_scalar;
       occ = ls.occ_scalar;
     }
