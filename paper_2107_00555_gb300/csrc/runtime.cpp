@@ -261,9 +261,10 @@ static void* dalloc(GraphImpl::Runtime& rt, size_t bytes) {
   return p;
 }
 
-// Allows a kernel its dynamic shared memory; CTAs resident per SM.
+// Allows a kernel its dynamic shared memory (48 KB are free only without static
+// shared memory beside it); CTAs resident per SM.
 static int prepare_function(CUfunction fn, const CodegenOut& code) {
-  if (code.smem_bytes > 48 * 1024)
+  if (code.smem_bytes > 0)
     check_cu(drv().funcSetAttribute(fn, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES,
                                     code.smem_bytes),
              "cuFuncSetAttribute(max dynamic smem)");
