@@ -276,14 +276,16 @@ struct Planner {
         g.groups[gi].kind == GroupKind::Map && computed_in(gi, a)) {
       const Group& M = g.groups[gi];
       bool ok = M.reds.empty() && M.shape == an.shape && axis_closure(M, gi, n.axis, due);
-      // binary64 maps with exp, sin and the like are bound by the FP64 pipe,
-      // which the map kernel keeps busier than a row tree: maps still to come
-      // then stay in its one pass (8063 x 140 binary64 columns 99 us against
-      // 168 in one kernel, 6751 x 1810 rows 784 against 848)
+      // binary64 maps with tanh, exp, sin and the like are bound by the FP64
+      // pipe, which the map kernel keeps busier than a row tree: maps still to
+      // come then stay in its one pass (sum of x^4 and maximum of tanh(x^4): the
+      // columns of 8063 x 140 53 us against 70 in one kernel, of 500 x 500 33
+      // against 66; of sin(x^4): 70 against 107 and 39 against 103)
       double cost = 0;
       for (int m : M.members) cost += op_cycles(g.nodes[m].op, an.dtype);
+      for (int m : due.maps) cost += op_cycles(g.nodes[m].op, an.dtype);
       if (!due.maps.empty() && !fmaps()) ok = false;  // (maps are not to be fused with one another)
-      if (an.dtype == DCP_F64 && !due.maps.empty() && cost > 12 * op_cycles(DCP_ADD, DCP_F64)) ok = false;
+      if (an.dtype == DCP_F64 && !due.maps.empty() && cost >= 8 * op_cycles(DCP_ADD, DCP_F64)) ok = false;
       if (ok && (int)due.loads.size() <= kMaxIO && (int)due.scalars.size() <= kMaxIO &&
           (int)due.reds.size() <= kMaxIO) {
         R.members = M.members;

@@ -59,3 +59,15 @@ def test_maps_stay_apart_unless_maps_are_to_be_fused():
     g.output(g.reduce(g.map("abs", [g.map("sub", [y, x])]), "max", axis=1))
     kinds = _groups(g, C.DCP_FUSE_SUBGRAPH)
     assert all(members <= 1 for _, members, _, _ in kinds)
+
+
+@pytest.mark.parametrize("op,together", [("abs", True), ("sqrt", False), ("tanh", False), ("sin", False)])
+def test_costly_binary64_maps_after_a_reduction_keep_their_own_kernel(op, together):
+    """Counted over all the maps: those planned with the first reduction and
+    those still to come."""
+    g = Graph()
+    y = g.map("square", [g.input("f64", SHAPE)])
+    g.output(g.reduce(y, "sum", axis=0))
+    g.output(g.reduce(g.map(op, [y]), "max", axis=0))
+    kinds = [k for k, _, _, _ in _groups(g)]
+    assert kinds == (["axis_reduce"] if together else ["map", "axis_reduce"])
