@@ -26,7 +26,7 @@
 //
 // The generated prefix defines DCP_T, DCP_THREADS, DCP_KNAME, DCP_NRED,
 // DCP_NLOAD, DCP_NSCALAR, DCP_VEC, DCP_AXMODE (0: vectors along inner, 1:
-// along R), dcp_red_op(r) and
+// along R), DCP_LONG (at least 64 elements along R), dcp_red_op(r) and
 //   void dcp_body(const T* ld, const T* sc, T* rv)
 //        the reduced operands (prologue maps fused) from one element's loads
 typedef DCP_T T;
@@ -38,7 +38,12 @@ constexpr int V = DCP_VEC;                   // elements per load
 constexpr int VO = DCP_AXMODE == 0 ? V : 1;  // outputs per thread
 constexpr int NL = DCP_ARR(DCP_NLOAD);
 constexpr int NQ = DCP_ARR(DCP_NRED);
-constexpr int UNR = V > 1 ? 2 : 8;           // loads in flight per thread and input
+// Loads in flight per thread and input.  A single input read element by element
+// takes eight (sums down 4096 x 4095 binary32: 27 us at four, 19 at eight);
+// with more inputs the values no longer fit the registers (the sum of six
+// arrays of that size: 98 us at four, 188 at eight).
+// (Short axes never fill eight, whose registers cost them warps.)
+constexpr int UNR = V > 1 ? 2 : (NL == 1 && DCP_LONG ? 8 : 4);
 
 // The V consecutive elements of every input at flat index gi.
 __device__ __forceinline__ void dcp_load_v(const DcpAxParams& p, long long gi, T (&ld)[NL][V]) {
