@@ -342,7 +342,8 @@ CodegenOut gen_axis_kernel(const GraphImpl& g, const Group& G, bool vec_ok) {
   os << "#define DCP_T " << dtype_cname(T) << "\n#define DCP_THREADS " << G.threads
      << "\n#define DCP_NRED " << G.reds.size() << "\n#define DCP_NLOAD " << G.loads.size()
      << "\n#define DCP_NSCALAR " << G.scalars.size() << "\n#define DCP_VEC " << vec
-     << "\n#define DCP_AXMODE " << axmode << "\n#define DCP_LONG " << (R >= 64 ? 1 : 0) << "\n";
+     << "\n#define DCP_AXMODE " << axmode << "\n#define DCP_RAGGED " << (axmode == 1 && R % vec != 0 ? 1 : 0)
+     << "\n#define DCP_LONG " << (R >= 64 ? 1 : 0) << "\n";
   os << red_op_fn(g, G.reds);
   os << "#include \"dcp_device.cuh\"\n";
   os << "__device__ __forceinline__ void dcp_body(const DCP_T* ld, const DCP_T* sc, DCP_T* rv) {\n";
