@@ -871,13 +871,21 @@ bool listed_star3(const std::vector<int32_t>& offs, int n) {
   return true;
 }
 
+// Can step s of the group be summed by the column kernel?
+bool column_step(const GraphImpl& g, const Group& G, int s) {
+  const Node& n = g.nodes[G.steps[s].node];
+  return G.dtype == DCP_F64 ? plan_sum3(G.dtype, G.offsets, n.weights, plan_defer(g, G, s)).pairs
+                            : listed_star3(G.offsets, n.npts());
+}
+
 // Warp-streamed columns of a 3-D star (k_stencil3d_col.cuh).
 static CodegenOut gen_column_kernel(const GraphImpl& g, const Group& G, int s0, int s1, int max_vec) {
   NameScope names;
   const int T = G.dtype, K = s1 - s0, C = stream_cols_per_lane(T);
   const bool first = s0 == 0, last = s1 == (int)G.steps.size();
   const bool f64 = T == DCP_F64;
-  if (!column_eligible(g, G)) fail(DCP_E_UNSUPPORTED, "3-D columns do not suit this stencil group");
+  for (int s = s0; s < s1; ++s)
+    if (!column_step(g, G, s)) fail(DCP_E_UNSUPPORTED, "3-D columns do not suit this stencil group");
   int vec = std::min(C, max_vec);
   while (G.shape.back() % vec != 0) vec /= 2;
   std::ostringstream os;
@@ -1219,12 +1227,8 @@ bool column_eligible(const GraphImpl& g, const Group& G) {
   if (G.kind != GroupKind::Stencil || G.shape.size() != 3 || !G.members.empty()) return false;
   if (G.radius[0] != 1 || G.radius[1] > 1 || G.radius[2] > 1) return false;
   if (G.shape[1] * G.shape[2] > 0x7fffffff) return false;  // offsets within a plane are 32-bit
-  for (int s = 0; s < (int)G.steps.size(); ++s) {
-    const Node& n = g.nodes[G.steps[s].node];
-    if (G.dtype == DCP_F64 ? !plan_sum3(G.dtype, G.offsets, n.weights, plan_defer(g, G, s)).pairs
-                           : !listed_star3(G.offsets, n.npts()))
-      return false;
-  }
+  for (int s = 0; s < (int)G.steps.size(); ++s)
+    if (!column_step(g, G, s)) return false;
   return true;
 }
 
