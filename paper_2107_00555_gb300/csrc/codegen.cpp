@@ -888,15 +888,18 @@ static CodegenOut gen_column_kernel(const GraphImpl& g, const Group& G, int s0, 
     if (!column_step(g, G, s)) fail(DCP_E_UNSUPPORTED, "3-D columns do not suit this stencil group");
   int vec = std::min(C, max_vec);
   while (G.shape.back() % vec != 0) vec /= 2;
+  // four warps share the ticket of a launch that reduces (see gen_stream_kernel),
+  // but where two steps of four rows need every register
+  const int threads = last && !G.reds.empty() && !f64 && K * G.cy < 8 ? 4 * G.threads : G.threads;
   std::ostringstream os;
   os << "// dcp 3-D column stencil kernel: " << K << " steps per launch, bc " << G.bc << "\n";
   os << "#define DCP_T " << dtype_cname(T) << "\n#define DCP_C " << C << "\n#define DCP_CY " << G.cy
      << "\n#define DCP_LX " << G.lx << "\n#define DCP_NSTEPS " << K << "\n#define DCP_R " << kColumnRing << "\n#define DCP_W "
      << column_width(G, K) << "\n#define DCP_VEC " << vec << "\n#define DCP_PAIRS " << (f64 ? 1 : 0)
-     << "\n#define DCP_BC " << G.bc << "\n#define DCP_THREADS " << G.threads << "\n#define DCP_LAST "
+     << "\n#define DCP_BC " << G.bc << "\n#define DCP_THREADS " << threads << "\n#define DCP_LAST "
      << (last ? 1 : 0) << "\n#define DCP_POST "
      << (last && (!G.post.empty() || !G.reds.empty() || G.stores.size() != 1) ? 1 : 0)
-     << "\n#define DCP_MINB " << std::max(1, G.min_ctas) << "\n#define DCP_NSTORE "
+     << "\n#define DCP_MINB " << std::max(1, G.min_ctas * G.threads / threads) << "\n#define DCP_NSTORE "
      << (last ? (int)G.stores.size() : 1) << "\n#define DCP_NRED " << (last ? (int)G.reds.size() : 0)
      << "\n#define DCP_NSCALAR " << G.scalars.size() << "\n";
   const Defer guard = first ? plan_defer(g, G, 0) : Defer();
@@ -962,10 +965,10 @@ static CodegenOut gen_column_kernel(const GraphImpl& g, const Group& G, int s0, 
   }
   os << km.table() << decl.str() << sums.str();
   os << "#include \"k_stencil3d_col.cuh\"\n";
-  out.threads = G.threads;
+  out.threads = threads;
   out.vec = vec;
   out.guard_max_input = guard.on ? guard.max_input : 0.0;
-  out.smem_bytes = G.threads / 32 * kColumnRing * (32 / G.lx * G.cy + 2 * K) * ((G.lx + 2) * C) * dtype_size(T);
+  out.smem_bytes = threads / 32 * kColumnRing * (32 / G.lx * G.cy + 2 * K) * ((G.lx + 2) * C) * dtype_size(T);
   out.source = finish("dcp_col3d", os.str());
   out.name = kname_of(out.source);
   return out;
@@ -997,6 +1000,12 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
   const int nin = std::max(1, nload);  // a prologue of broadcast scalars loads no array
   int threads = G.threads, ring = 8;  // a power of two
   while (ring < 8 * G.prefetch) ring *= 2;
+  // Every CTA of a launch that reduces takes a ticket, about 7 ns each, one
+  // after the other: four binary32 warps share one (a step of 1000 x 1001 with
+  // its maximum 18.5 -> 11 us).  The FP64 pipes would be shared out too
+  // unevenly (3000 x 3100: 160 us in CTAs of two warps, 209 in CTAs of eight).
+  if (last && !G.reds.empty() && T == DCP_F32 && !g.options.count(DCP_OPT_STREAM_THREADS))
+    threads = std::max(threads, 128);
   auto smem = [&] { return threads / 32 * nin * ring * 512; };
   while (smem() > 192 * 1024 && ring > 4) ring /= 2;
   while (smem() > 192 * 1024 && threads > 32) threads = threads / 64 * 32;
@@ -1012,7 +1021,7 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
      << "\n#define DCP_VEC " << vec << "\n";
   const Defer guard = first ? plan_defer(g, G, 0) : Defer();
   os << "#define DCP_GUARD " << (guard.on ? 1 : 0) << "\n";
-  if (G.min_ctas > 0) os << "#define DCP_MINB " << G.min_ctas << "\n";
+  if (G.min_ctas > 0) os << "#define DCP_MINB " << std::max(1, G.min_ctas * G.threads / threads) << "\n";
   os << red_op_fn(g, last ? G.reds : std::vector<int>{});
   os << "#include \"dcp_device.cuh\"\n";
   if (!batch) {

@@ -1,0 +1,32 @@
+"""Which kernel form, depth and work split the planner gives stencil programs
+whose best form is not the one their family usually takes (no GPU needed)."""
+import pytest
+
+from paper_2107_00555_gb300 import _capi as C
+from paper_2107_00555_gb300 import Graph, programs
+
+STAR2 = [(0, 0), (0, -1), (0, 1), (-1, 0), (1, 0), (0, -2), (0, 2), (-2, 0), (2, 0)]
+W2 = [0.4, 0.1, 0.1, 0.1, 0.1, 0.05, 0.05, 0.05, 0.05]
+
+
+def _stencil(shape, dtype, bc, steps, offs=programs.FIVE_POINT, w=programs.FIVE_WEIGHTS, arrays=1,
+             reduced=False, flags=C.DCP_FUSE_ALL):
+    g = Graph()
+    u = g.input(dtype, shape)
+    for _ in range(arrays - 1):
+        u = g.map("add", [g.map("mul_s", [u], 0.5), g.input(dtype, shape)])
+    u = g.stencil(u, offs, w, bc, steps)
+    g.output(u)
+    if reduced:
+        g.output(g.reduce(u, "max"))
+    g.fuse(flags)
+    plan = g.plan()
+    return plan["groups"][0], plan["launches"]
+
+
+def test_launches_that_reduce_share_tickets_between_binary32_warps():
+    grp, launches = _stencil((1000, 1001), "f32", "zero", 14, reduced=True)
+    assert grp["kernel_form"] == "stream" and grp["threads"] == 32
+    assert [l["threads"] for l in launches] == [32] * (len(launches) - 1) + [128]
+    _, launches = _stencil((3000, 3100), "f64", "zero", 1, reduced=True)
+    assert launches[-1]["threads"] == 64
