@@ -989,6 +989,8 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
   int vec = 0;
   if (!batch)
     for (vec = std::min(C, max_vec); G.shape.back() % vec != 0;) vec /= 2;
+  const bool exact = stream_exact(G);
+  if (exact) vec = 1;
   std::ostringstream os;
   os << "// dcp warp-stream stencil kernel: " << nsteps << " steps per launch, bc " << G.bc << ", "
      << nd << "-D" << (batch ? ", batched" : "") << "\n";
@@ -998,8 +1000,9 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
   // 512 bytes each; fewer rows, then fewer warps per CTA where 192 KB is short
   const int nload = pro ? (int)G.loads.size() : 1;
   const int nin = std::max(1, nload);  // a prologue of broadcast scalars loads no array
-  int threads = G.threads, ring = 8;  // a power of two
-  while (ring < 8 * G.prefetch) ring *= 2;
+  // A 1-D array's items are one row each.
+  int threads = G.threads, ring = nd == 1 ? 4 : 8;  // a power of two
+  for (const int rows = ring * G.prefetch; ring < rows;) ring *= 2;
   // Every CTA of a launch that reduces takes a ticket, about 7 ns each, one
   // after the other: four binary32 warps share one (a step of 1000 x 1001 with
   // its maximum 18.5 -> 11 us).  The FP64 pipes would be shared out too
@@ -1018,6 +1021,7 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
      << (last && (!G.post.empty() || !G.reds.empty() || G.stores.size() != 1) ? 1 : 0) << "\n";
   os << "#define DCP_RX " << rx << "\n#define DCP_RY " << ry << "\n#define DCP_NSTEPS " << nsteps
      << "\n#define DCP_R " << ring << "\n#define DCP_W " << stream_width(G, nsteps)
+     << "\n#define DCP_HX " << (exact ? nsteps * rx : (nsteps * rx + C - 1) / C * C)
      << "\n#define DCP_VEC " << vec << "\n";
   const Defer guard = first ? plan_defer(g, G, 0) : Defer();
   os << "#define DCP_GUARD " << (guard.on ? 1 : 0) << "\n";

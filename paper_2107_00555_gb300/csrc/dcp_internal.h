@@ -295,8 +295,14 @@ inline int stream_cols_per_lane(int dtype) { return dtype == DCP_F64 || dtype ==
 // Columns a warp writes per row in a launch of nsteps steps: the strip minus
 // its halos, the left one rounded up and the width rounded down to whole
 // vectors, so that strips start on vector boundaries of an aligned row.
+// Binary64 1-D arrays, which the FP64 pipe bounds, take strips of any width and
+// single elements instead.
+inline bool stream_exact(const Group& G) {
+  return G.kind == GroupKind::Stencil && G.shape.size() == 1 && G.dtype == DCP_F64;
+}
 inline int stream_width(const Group& G, int nsteps) {
   const int C = stream_cols_per_lane(G.dtype), h = nsteps * G.radius[2];
+  if (stream_exact(G)) return 32 * C - 2 * h;
   return (32 * C - (h + C - 1) / C * C - h) / C * C;
 }
 inline int default_stream_threads(const Group& G) {

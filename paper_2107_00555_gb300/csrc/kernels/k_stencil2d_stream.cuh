@@ -30,7 +30,9 @@
 // DCP_W columns starting at a multiple of C, its first lane HX (the halo
 // rounded up to whole vectors) columns to the left, so that rows of a 16-byte
 // multiple are read and written in whole vectors; other row lengths fall back
-// to the widest access that divides them.
+// to the widest access that divides them.  Strips of 1-D binary64 arrays are
+// as wide as their halos allow and go element by element: the FP64 pipe bounds
+// them, and vectors cost a step 2 of 62 columns.
 //
 // Boundaries: ZERO clears the columns (CHECK strips) and rows outside the
 // array at every level; FIXED_RING lets the sums of ring cells carry the
@@ -43,7 +45,7 @@
 //
 // The generated prefix defines DCP_T, DCP_C, DCP_RX, DCP_RY, DCP_NSTEPS,
 // DCP_BC, DCP_THREADS, DCP_KNAME, DCP_BATCH, DCP_LAST, DCP_R, DCP_GUARD, DCP_MINB,
-// DCP_W, DCP_VEC (elements per access, 0: per instance), DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions after the last step), DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
+// DCP_W, DCP_HX, DCP_VEC (elements per access, 0: per instance), DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions after the last step), DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
 //   T    dcp_pro(const T (&ld)[DCP_NIN], const T* sc)     input maps on the loaded values
 //   struct DcpRow<L>::run<RINGM>(a, st, out, km, rm)      arrival of row a in level L+1
 //   T    dcp_epi<L>(T v)                 epilogue maps fused after step L
@@ -64,10 +66,10 @@ constexpr int C = DCP_C;
 constexpr int RY = DCP_RY;
 constexpr int NST = DCP_ARR(2 * RY);               // partial sums per column and level
 constexpr int SPAN = 32 * C;                       // columns held by a warp
-constexpr int HX = (K * DCP_RX + C - 1) / C * C;   // left halo, whole vectors
+constexpr int HX = DCP_HX;                         // left halo, whole vectors (DCP_VEC 1: any)
 constexpr int W = DCP_W;                           // columns written by a warp
-static_assert(W > 0 && W % C == 0 && HX + W + K * DCP_RX <= SPAN,
-              "strip too narrow for the number of steps");
+static_assert(W > 0 && HX + W + K * DCP_RX <= SPAN, "strip too narrow for the number of steps");
+static_assert(DCP_VEC == 1 || (W % C == 0 && HX % C == 0), "strips start on vector boundaries");
 constexpr int RING = DCP_BC == DCP_BC_FIXED_RING ? RY : 0;  // ring rows
 
 constexpr int R = DCP_R;                           // rows of a warp's ring
@@ -228,10 +230,15 @@ __device__ __forceinline__ void dcp_src(const T* (&src)[DCP_NIN], int row, const
   for (int l = 0; l < DCP_NLOAD; ++l) src[l] = it.in[l] + at;
 }
 
-// Requests input row j with its boundary tests (zeros outside the array).
+// Requests input row j with its boundary tests (zeros outside the array).  An
+// item of a 1-D array is one row: the rows after it are only counted.
 template <bool CHECK>
 __device__ __forceinline__ void dcp_request_checked(unsigned so, int j, const DcpItem& it,
                                                     const DcpCols& cols) {
+  if (RY == 0 && j >= it.y1) {
+    dcp_commit();
+    return;
+  }
   const bool inside = (unsigned)j < (unsigned)it.ny;
   const T* src[DCP_NIN];
   dcp_src<CHECK>(src, DCP_BC == DCP_BC_PERIODIC ? dcp_wrap(j, it.ny) : (inside ? j : 0), it);
