@@ -435,16 +435,27 @@ struct Defer {
   double max_input = 0.0;     // largest finite |input| the run keeps finite
 };
 
-bool defer_ratios(const std::vector<double>& w, std::vector<double>& ratio, double& f_out,
-                  double& gsum) {
+// f: the most frequent nonzero weight; of equally frequent ones, on 2 axes, one
+// with a point in the neighbourhood's first row, where the row-by-row sums
+// start (a 9-point star of radius 2, sides 0.1 and 0.05, then takes 8
+// operations instead of 9).
+bool defer_ratios(const Node& n, std::vector<double>& ratio, double& f_out, double& gsum) {
+  const std::vector<double>& w = n.weights;
   const int P = (int)w.size();
   double f = 0.0;
   int best = 0;
-  for (int k = 0; k < P; ++k) {  // f: the most frequent nonzero weight
+  auto first_row = [&](double v) {
+    int top = n.offsets[0];
+    bool in = false;
+    for (int k = 0; k < P; ++k) top = std::min(top, n.offsets[2 * k]);
+    for (int k = 0; k < P; ++k) in = in || (w[k] == v && n.offsets[2 * k] == top);
+    return in;
+  };
+  for (int k = 0; k < P; ++k) {
     if (w[k] == 0.0) continue;
     int c = 0;
     for (int j = 0; j < P; ++j) c += w[j] == w[k];
-    if (c > best) best = c, f = w[k];
+    if (c > best || (c == best && n.ndim() == 2 && !first_row(f) && first_row(w[k]))) best = c, f = w[k];
   }
   if (f == 0.0 || !std::isfinite(f)) return false;
   ratio.assign(P, 0.0);
@@ -468,7 +479,7 @@ int defer_chunk_steps(const Node& n) {
   if (n.dtype != DCP_F64 || (n.bc != DCP_BC_ZERO && n.bc != DCP_BC_PERIODIC)) return 0;
   std::vector<double> r;
   double f = 0.0, gsum = 0.0;
-  if (!defer_ratios(n.weights, r, f, gsum)) return 0;
+  if (!defer_ratios(n, r, f, gsum)) return 0;
   if (gsum <= 1.0) return INT32_MAX;
   const int D = (int)std::floor(32.0 / std::log2(gsum));
   return D >= 2 ? D : 0;
@@ -497,7 +508,7 @@ Defer plan_defer(const GraphImpl& g, const Group& G, int s) {
   if (L < 2) return d;
   std::vector<double> r;
   double f = 0.0, gsum = 0.0;
-  if (!defer_ratios(n.weights, r, f, gsum)) return d;
+  if (!defer_ratios(n, r, f, gsum)) return d;
   const int Dmax = defer_chunk_steps(n);
   if (Dmax == 0) return d;
   const int D = std::min(L, Dmax);

@@ -50,3 +50,19 @@ def test_1d_streams_same_bits_as_tiles(bc, dtype):
             for depth in (1, 2, 3, 4):
                 for off in (False, True):
                     assert _run(x, offs, w, bc, 7, 1, depth, off) == ref, (n, radius, depth, off)
+
+
+@pytest.mark.parametrize("bc", ["zero", "periodic"])
+@pytest.mark.parametrize("shape", [(37, 130), (300, 257)])
+def test_radius_two_star_on_its_deferred_weight(shape, bc):
+    x = inputs.uniform(shape, -1.0, 1.0, 5, np.float64)
+    ref = _run(x, STAR2, W2, bc, 9, 0, 1)
+    for kernel, depth in ((0, 3), (1, 1), (1, 2), (1, 4)):
+        assert _run(x, STAR2, W2, bc, 9, kernel, depth) == ref
+    u = x
+    for _ in range(9):
+        p = np.pad(u, 2, mode="wrap" if bc == "periodic" else "constant")
+        u = sum(c * p[2 + dy:2 + dy + shape[0], 2 + dx:2 + dx + shape[1]] for c, (dy, dx) in zip(W2, STAR2))
+    got = np.frombuffer(ref[0]).reshape(shape)
+    # 9 convex steps of at most 10 roundings each on either side
+    assert np.abs(got - u).max() <= 9 * 20 * np.finfo(np.float64).eps

@@ -30,3 +30,11 @@ def test_launches_that_reduce_share_tickets_between_binary32_warps():
     assert [l["threads"] for l in launches] == [32] * (len(launches) - 1) + [128]
     _, launches = _stencil((3000, 3100), "f64", "zero", 1, reduced=True)
     assert launches[-1]["threads"] == 64
+
+
+def test_deferred_weight_is_one_of_the_first_row():
+    """Sides 0.1 and 0.05 are equally frequent; the row sums start at 0.05's
+    point, which then needs no multiply."""
+    _, launches = _stencil((1000, 1001), "f64", "zero", 3, STAR2, W2)
+    scales = [s for l in launches for s in l["deferred_scales"]]
+    assert scales[:2] == [1, 1] and scales[2] == pytest.approx(0.05 ** 3, rel=1e-15)
