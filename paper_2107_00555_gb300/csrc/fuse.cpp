@@ -585,6 +585,9 @@ struct Planner {
     return it == g.options.end() ? def : it->second;
   }
 
+  // The planner runs without a GPU: a GB300's SMs and their warp schedulers.
+  static constexpr int64_t kSMs = 152, kSchedulers = 4 * kSMs;
+
   // Issue cycles of one operation on the C columns a lane holds (binary64
   // operations cost the FP64 pipe 64 cycles per warp and scheduler).
   double op_cycles(int op, int dtype) const {
@@ -643,7 +646,7 @@ struct Planner {
     // where both arrays stay in L2
     const double mem = bytes / (bytes > 100e6 ? 3237.0 : 6500.0);
     double best = 1e300;
-    const int64_t slots = 152 * 4;
+    const int64_t slots = kSchedulers;
     for (int n = 1; n <= 4; ++n) {
       const int64_t segs = std::max<int64_t>(1, std::min<int64_t>(ny, n * slots / strips));
       const int64_t sg = (ny + segs - 1) / segs;
@@ -660,7 +663,7 @@ struct Planner {
   }
 
   // Cycles of one batched launch of K steps with seg rows per work item: the
-  // issue of every item's rows over the 608 schedulers plus half an item's
+  // issue of every item's rows over the GPU's schedulers plus half an item's
   // time for the uneven end, at least one item's latency.  (4096 binary32
   // instances of 32^2 to 512^2, 20 steps at 5 per launch: 32, 64, 128 and 256
   // rows took 2.51, 2.23, 2.18 and 2.24 ms.)
@@ -686,8 +689,8 @@ struct Planner {
       longest = std::max(longest, std::min<int64_t>(ny, seg) + 2 * K * ry);
       bytes += 2.0 * ny * nx * dtype_size(G.dtype);
     }
-    const double n = std::min(4.0, items / 608.0);
-    const double c = std::max(rows * issue / 608 + 0.5 * longest * std::max(latency, n * issue),
+    const double n = std::min(4.0, items / (double)kSchedulers);
+    const double c = std::max(rows * issue / kSchedulers + 0.5 * longest * std::max(latency, n * issue),
                               longest * latency);
     return std::max(c, bytes / (bytes > 100e6 ? 3237.0 : 6500.0));
   }
@@ -699,7 +702,7 @@ struct Planner {
   double tile_cycles(const Group& G, int K, int ty, int tx) const {
     const int64_t ny = G.shape[0], nx = G.shape[1];
     const int64_t tiles = ((ny + ty - 1) / ty) * ((nx + tx - 1) / tx);
-    const int64_t per = (tiles + 151) / 152;  // tiles of one SM
+    const int64_t per = (tiles + kSMs - 1) / kSMs;  // tiles of one SM
     const int pts = (int)G.offsets.size() / 3;
     double t = 0, epi = 0;
     for (const StepDesc& st : G.steps)
@@ -746,7 +749,7 @@ struct Planner {
     // (binary32: 63 instructions per cell, 3.84e-3 cycles of the whole GPU)
     const double padded = (double)nz * ((ny + 7) / 8 * 8) * ((nx + 31) / 32 * 32);
     best = 0.95 * S *
-           ((f64 ? std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / 304 + 3000)
+           ((f64 ? std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / (2 * kSMs) + 3000)
                  : std::max(mem, 3.84e-3 * padded * (0.6 + 0.4 * pts / 7 + epi / 252) + 5000)) + 6200);
     const int lx0 = G.lx, cy0 = G.cy;
     const bool odd = nx % 4 != 0;
@@ -771,11 +774,11 @@ struct Planner {
           const int nmax = f64 && cy == 8 ? 2 : 3;
           for (int n = 1; n <= nmax; ++n)
             for (int wv = 1; wv <= (n == nmax ? 16 : 1); ++wv) {  // whole waves of the resident warps
-              const int64_t segs = (int64_t)wv * n * 608 / (strips * blocks);
+              const int64_t segs = (int64_t)wv * n * kSchedulers / (strips * blocks);
               if (segs < 1) continue;
               const int64_t sg = (nz + std::min(segs, nz) - 1) / std::min(segs, nz);
               const int64_t items = strips * blocks * ((nz + sg - 1) / sg);
-              const int64_t per = (items + 607) / 608;
+              const int64_t per = (items + kSchedulers - 1) / kSchedulers;
               const int64_t waves = (per + n - 1) / n;
               // (one warp alone keeps its scheduler's FP64 pipe busy 70 % of the time)
               const int64_t nn = std::min<int64_t>(per, n);
@@ -785,9 +788,9 @@ struct Planner {
               if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
               if (segs >= nz) break;
             }
-          if (strips * blocks > 16 * nmax * 608) {  // wide grids: long columns
+          if (strips * blocks > 16 * nmax * kSchedulers) {  // wide grids: long columns
             const int64_t sg = std::min<int64_t>(nz, 64);
-            const double c = ((double)strips * blocks * nz / sg / 608 * (sg + ends) * issue + 6200) * ((S + K - 1) / K);
+            const double c = ((double)strips * blocks * nz / sg / kSchedulers * (sg + ends) * issue + 6200) * ((S + K - 1) / K);
             if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
           }
         }
@@ -850,8 +853,17 @@ struct Planner {
           !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS)) {
         for (int most = 1; most <= std::min(S, 12); ++most) {
           const int K = free_depth ? even(most) : G.depth;
-          for (int tx : {16, 32})
-            for (int ty : {4, 8, 12, 14, 16, 24, 32}) {
+          for (int tx : {16, 32}) {
+            std::vector<int> heights = {4, 8, 12, 16, 24, 32};
+            // heights that give every SM the same number of tiles, one or two
+            // (256 rows in 8 strips: 14, 152 tiles; 16 rows would leave 24 SMs idle)
+            const int64_t strips = (G.shape[1] + tx - 1) / tx;
+            for (int per : {1, 2})
+              if (per * kSMs >= strips) {
+                const int64_t rows = per * kSMs / strips, ty = (G.shape[0] + rows - 1) / rows;
+                if (ty >= 4 && ty <= 32) heights.push_back((int)ty);
+              }
+            for (int ty : heights) {
               const long smem = 2L * (ty + 2 * K * G.radius[1]) * (tx + 2 * K * G.radius[2]) * dtype_size(G.dtype);
               if (smem > 96 * 1024) continue;
               const double c = total(tile_cycles(G, K, ty, tx), K) + 0.3 * launch * ((S + K - 1) / K);
@@ -863,6 +875,7 @@ struct Planner {
                 G.tile[2] = tx;
               }
             }
+          }
           if (!free_depth) break;
         }
       }

@@ -24,6 +24,12 @@ def _stencil(shape, dtype, bc, steps, offs=programs.FIVE_POINT, w=programs.FIVE_
     return plan["groups"][0], plan["launches"]
 
 
+def test_tile_heights_follow_the_number_of_sms():
+    """512 rows in 16 strips: two tiles for each of 152 SMs."""
+    grp, _ = _stencil((512, 512), "f64", "zero", 10)
+    assert grp["kernel_form"] == "tile" and grp["tile"][1:] == [27, 32]
+
+
 def test_launches_that_reduce_share_tickets_between_binary32_warps():
     grp, launches = _stencil((1000, 1001), "f32", "zero", 14, reduced=True)
     assert grp["kernel_form"] == "stream" and grp["threads"] == 32
