@@ -613,6 +613,14 @@ struct Planner {
     return run ? std::max(1, pts == 5 ? pts - 2 : pts - 1) : pts;
   }
 
+  // Issue cycles of a step's epilogue maps, averaged over the steps.
+  double epi_cycles(const Group& G) const {
+    double c = 0;
+    for (const StepDesc& st : G.steps)
+      for (int e : st.epi) c += op_cycles(g.nodes[e].op, G.dtype);
+    return c / (double)G.steps.size();
+  }
+
   // Cycles of one launch of K steps of the warp-stream kernel, and the rows
   // per work item that give them: nw warps per scheduler (4 per SM) stream
   // seg + 2 K ry rows each, a row taking the larger of its latency and the
@@ -635,10 +643,7 @@ struct Planner {
       issue = K * (7.0 + 4.0 * pts) + 42;
       latency = 130.0 + 45.0 * K;
     }
-    double epi = 0;
-    for (const StepDesc& st : G.steps)
-      for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
-    issue += K * epi / (double)G.steps.size();
+    issue += K * epi_cycles(G);
     for (int m : G.members) issue += op_cycles(g.nodes[m].op, G.dtype);
     const int64_t cells = ny * nx;
     const double bytes = 2.0 * cells * dtype_size(G.dtype);
@@ -696,24 +701,31 @@ struct Planner {
   }
 
   // Cycles of one launch of K steps of the shared-memory tile kernel (256
-  // threads per CTA), fitted to the same runs: a step takes about 290 cycles
-  // per 256 cells of its region (binary32, two CTAs per SM in parallel) or, on
-  // binary64, 1200 plus the region's operations at 2 per clock.
-  double tile_cycles(const Group& G, int K, int ty, int tx) const {
-    const int64_t ny = G.shape[0], nx = G.shape[1];
-    const int64_t tiles = ((ny + ty - 1) / ty) * ((nx + tx - 1) / tx);
+  // threads per CTA) on `tiles` tiles.  Binary32: about 290 cycles per step and
+  // 256 cells of the region, two CTAs per SM in parallel (fitted to 24 steps
+  // on 64^2 .. 512^2).  Binary64: per tile 350 cycles and the operations of
+  // its regions at 2 per clock, 0.7 operations per cell more than the sum's and
+  // 5 % over, and per step 1000 cycles of latency, 1200 where the SM has no
+  // other tile (within 10 %: 5-, 9- and 13-point steps of radius 1 and 2, one
+  // and two per launch, on 500 x 513 .. 3000 x 3100; 5 and 10 steps on 256^2 .. 512^2).
+  double tile_cycles(const Group& G, int K, int ty, int tx, int64_t tiles) const {
     const int64_t per = (tiles + kSMs - 1) / kSMs;  // tiles of one SM
     const int pts = (int)G.offsets.size() / 3;
-    double t = 0, epi = 0;
-    for (const StepDesc& st : G.steps)
-      for (int e : st.epi) epi += op_cycles(g.nodes[e].op, G.dtype);
-    epi /= (double)G.steps.size();
+    const int ry = G.radius[1], rx = G.radius[2];
+    const bool f64 = G.dtype == DCP_F64;
+    const double epi = epi_cycles(G), parallel = std::max(1.0, per / 2.0);
+    const double ops = f64 ? std::min(pts, (int)step_ops64(G) + 1) + 0.7 + epi / 128 : 0;
+    double t = 0;
     for (int s = 0; s < K; ++s) {
-      const double cells = (double)(ty + 2 * (K - 1 - s) * G.radius[1]) * (tx + 2 * (K - 1 - s) * G.radius[2]);
-      if (G.dtype == DCP_F64) t += 1200 + per * cells * (std::min(pts, (int)step_ops64(G) + 1) + epi / 128) / 2;
-      else t += std::max(1.0, per / 2.0) * (290.0 * pts / 5 + 0.6 * epi) * std::ceil(cells / 256);
+      const double cells = (double)(ty + 2 * (K - 1 - s) * ry) * (tx + 2 * (K - 1 - s) * rx);
+      if (f64) t += (per == 1 ? 1200 : 1000) + per * cells * 1.05 * ops / 2;
+      else t += parallel * (290.0 * pts / 5 + 0.6 * epi) * std::ceil(cells / 256);
     }
+    if (f64) t += per * 350;
     return t;
+  }
+  int64_t tiles_of(const std::vector<int64_t>& shape, int ty, int tx) const {
+    return ((shape[0] + ty - 1) / ty) * ((shape[1] + tx - 1) / tx);
   }
 
   // 3-D stars without a prologue run as warp-streamed columns where those are
@@ -848,9 +860,9 @@ struct Planner {
         }
       // Small grids run faster in shared-memory tiles, where every cell of a
       // step is in flight at once (256^2 binary64, 24 steps: 46 us against 91;
-      // 64^2 binary32: 17 against 25); from 512^2 on the stream wins.
-      if (nd == 2 && cells <= 512 * 512 && !has(DCP_OPT_STENCIL_KERNEL) && !has(DCP_OPT_TILE_X) &&
-          !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS)) {
+      // 64^2 binary32: 17 against 25).  From 512^2 on the stream wins.
+      if (nd == 2 && cells <= 512 * 512 && !has(DCP_OPT_STENCIL_KERNEL) &&
+          !has(DCP_OPT_TILE_X) && !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS)) {
         for (int most = 1; most <= std::min(S, 12); ++most) {
           const int K = free_depth ? even(most) : G.depth;
           for (int tx : {16, 32}) {
@@ -866,7 +878,8 @@ struct Planner {
             for (int ty : heights) {
               const long smem = 2L * (ty + 2 * K * G.radius[1]) * (tx + 2 * K * G.radius[2]) * dtype_size(G.dtype);
               if (smem > 96 * 1024) continue;
-              const double c = total(tile_cycles(G, K, ty, tx), K) + 0.3 * launch * ((S + K - 1) / K);
+              const int64_t tiles = tiles_of(G.shape, ty, tx);
+              const double c = total(tile_cycles(G, K, ty, tx, tiles), K) + 0.3 * launch * ((S + K - 1) / K);
               if (c < best) {
                 best = c;
                 var = 0;

@@ -24,6 +24,12 @@ def _stencil(shape, dtype, bc, steps, offs=programs.FIVE_POINT, w=programs.FIVE_
     return plan["groups"][0], plan["launches"]
 
 
+def test_one_step_on_a_small_binary64_grid_takes_large_tiles():
+    """4 x 16 cells keep a quarter of a CTA's threads busy."""
+    grp, _ = _stencil((500, 513), "f64", "periodic", 1)
+    assert grp["tile"][1] * grp["tile"][2] >= 512
+
+
 def test_tile_heights_follow_the_number_of_sms():
     """512 rows in 16 strips: two tiles for each of 152 SMs."""
     grp, _ = _stencil((512, 512), "f64", "zero", 10)
