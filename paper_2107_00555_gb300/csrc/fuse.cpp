@@ -860,27 +860,36 @@ struct Planner {
         }
       // Small grids run faster in shared-memory tiles, where every cell of a
       // step is in flight at once (256^2 binary64, 24 steps: 46 us against 91;
-      // 64^2 binary32: 17 against 25).  From 512^2 on the stream wins.
-      if (nd == 2 && cells <= 512 * 512 && !has(DCP_OPT_STENCIL_KERNEL) &&
+      // 64^2 binary32: 17 against 25).  From 512^2 on the stream wins, but for
+      // periodic binary64 grids: a step whose sums share no pairs pays for the
+      // strip's halo columns (1000 x 1001, 9 points of radius 2, 7 steps: 191 us
+      // streamed, 156 in tiles) and a narrow one for idle lanes.
+      const bool small = cells <= 512 * 512, f64 = G.dtype == DCP_F64;
+      const bool periodic = G.bc == DCP_BC_PERIODIC;
+      if (nd == 2 && (small || (f64 && periodic)) && !has(DCP_OPT_STENCIL_KERNEL) &&
           !has(DCP_OPT_TILE_X) && !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS)) {
-        for (int most = 1; most <= std::min(S, 12); ++most) {
+        for (int most = 1; most <= std::min(S, small ? 12 : 4); ++most) {
           const int K = free_depth ? even(most) : G.depth;
-          for (int tx : {16, 32}) {
-            std::vector<int> heights = {4, 8, 12, 16, 24, 32};
-            // heights that give every SM the same number of tiles, one or two
-            // (256 rows in 8 strips: 14, 152 tiles; 16 rows would leave 24 SMs idle)
-            const int64_t strips = (G.shape[1] + tx - 1) / tx;
-            for (int per : {1, 2})
-              if (per * kSMs >= strips) {
-                const int64_t rows = per * kSMs / strips, ty = (G.shape[0] + rows - 1) / rows;
-                if (ty >= 4 && ty <= 32) heights.push_back((int)ty);
-              }
+          for (int tx : small ? std::vector<int>{16, 32} : std::vector<int>{32}) {
+            std::vector<int> heights = {16, 32};
+            if (small) {
+              heights = {4, 8, 12, 16, 24, 32};
+              // heights that give every SM the same number of tiles, one or two
+              // (256 rows in 8 strips: 14, 152 tiles; 16 rows would leave 24 SMs idle)
+              const int64_t strips = (G.shape[1] + tx - 1) / tx;
+              for (int per : {1, 2})
+                if (per * kSMs >= strips) {
+                  const int64_t rows = per * kSMs / strips, ty = (G.shape[0] + rows - 1) / rows;
+                  if (ty >= 4 && ty <= 32) heights.push_back((int)ty);
+                }
+            }
             for (int ty : heights) {
               const long smem = 2L * (ty + 2 * K * G.radius[1]) * (tx + 2 * K * G.radius[2]) * dtype_size(G.dtype);
               if (smem > 96 * 1024) continue;
               const int64_t tiles = tiles_of(G.shape, ty, tx);
               const double c = total(tile_cycles(G, K, ty, tx, tiles), K) + 0.3 * launch * ((S + K - 1) / K);
-              if (c < best) {
+              // (on large grids more than two steps only for a gain the model resolves)
+              if (c < best * (small || K <= 2 || var == 1 ? 1.0 : 0.97)) {
                 best = c;
                 var = 0;
                 G.depth = K;

@@ -24,6 +24,22 @@ def _stencil(shape, dtype, bc, steps, offs=programs.FIVE_POINT, w=programs.FIVE_
     return plan["groups"][0], plan["launches"]
 
 
+def test_periodic_binary64_sums_without_shared_pairs_run_in_tiles():
+    grp, _ = _stencil((1000, 1001), "f64", "periodic", 7, STAR2, W2)
+    assert grp["kernel_form"] == "tile" and grp["tile"][1:] == [32, 32]
+    grp, _ = _stencil((1000, 1001), "f64", "periodic", 1)
+    assert grp["kernel_form"] == "tile"
+    # a long run of 5-point averages, which share their pairs, streams
+    grp, _ = _stencil((2047, 2051), "f64", "periodic", 20)
+    assert grp["kernel_form"] == "stream"
+
+
+def test_narrow_periodic_binary64_grids_run_in_tiles():
+    for shape in ((1000000, 4), (1000000, 1)):
+        grp, _ = _stencil(shape, "f64", "periodic", 10)
+        assert grp["kernel_form"] == "tile"
+
+
 def test_one_step_on_a_small_binary64_grid_takes_large_tiles():
     """4 x 16 cells keep a quarter of a CTA's threads busy."""
     grp, _ = _stencil((500, 513), "f64", "periodic", 1)
