@@ -613,6 +613,17 @@ struct Planner {
     return run ? std::max(1, pts == 5 ? pts - 2 : pts - 1) : pts;
   }
 
+  // Input arrays of a stencil group, and issue cycles of its prologue per row
+  // of a warp (binary64: a product and the add that takes it are one
+  // instruction, 0.6 per map).
+  int64_t arrays_in(const Group& G) const {
+    return G.members.empty() ? 1 : std::max<int64_t>(1, (int64_t)G.loads.size());
+  }
+  double pro_cycles(const Group& G) const {
+    double c = 0;
+    for (int m : G.members) c += op_cycles(g.nodes[m].op, G.dtype);
+    return G.dtype == DCP_F64 ? 0.6 * c : c;
+  }
   // Issue cycles of a step's epilogue maps, averaged over the steps.
   double epi_cycles(const Group& G) const {
     double c = 0;
@@ -629,7 +640,8 @@ struct Planner {
   // cycles per level and 42 per row with a latency of 45 per level and 130
   // per row; binary64 is bound by the FP64 pipe (p operations on 2 columns),
   // with a latency of 500 per level and 300 per row.
-  double stream_cycles(const Group& G, int K, int64_t& seg, int& nw) const {
+  // With `pro` the launch evaluates the group's prologue.
+  double stream_cycles(const Group& G, int K, bool pro, int64_t& seg, int& nw) const {
     const int64_t ny = G.shape.size() == 2 ? G.shape[0] : 1, nx = G.shape.back();
     const int ry = G.shape.size() == 2 ? G.radius[1] : 0;
     const int W = stream_width(G, K);
@@ -644,7 +656,8 @@ struct Planner {
       latency = 130.0 + 45.0 * K;
     }
     issue += K * epi_cycles(G);
-    for (int m : G.members) issue += op_cycles(g.nodes[m].op, G.dtype);
+    const int64_t inputs = pro ? arrays_in(G) : 1;
+    if (pro) issue += pro_cycles(G);
     const int64_t cells = ny * nx;
     const double bytes = 2.0 * cells * dtype_size(G.dtype);
     // 3237 bytes per clock from HBM (6.7 TB/s at 2.07 GHz), about twice that
@@ -652,8 +665,10 @@ struct Planner {
     const double mem = bytes / (bytes > 100e6 ? 3237.0 : 6500.0);
     double best = 1e300;
     const int64_t slots = kSchedulers;
-    for (int n = 1; n <= 4; ++n) {
-      const int64_t segs = std::max<int64_t>(1, std::min<int64_t>(ny, n * slots / strips));
+    // the rows in flight of every input take shared memory (227 KB per SM)
+    const int64_t resident = kSMs * std::max<int64_t>(1, 227 * 1024 / (inputs * 8 * 512));
+    for (int n = 1; n <= 4 && (n == 1 || n * slots <= resident); ++n) {
+      const int64_t segs = std::max<int64_t>(1, std::min<int64_t>(ny, std::min(n * slots, resident) / strips));
       const int64_t sg = (ny + segs - 1) / segs;
       const int64_t items = strips * ((ny + sg - 1) / sg);
       const int64_t per = (items + slots - 1) / slots;  // warps one scheduler runs
@@ -707,8 +722,9 @@ struct Planner {
   // its regions at 2 per clock, 0.7 operations per cell more than the sum's and
   // 5 % over, and per step 1000 cycles of latency, 1200 where the SM has no
   // other tile (within 10 %: 5-, 9- and 13-point steps of radius 1 and 2, one
-  // and two per launch, on 500 x 513 .. 3000 x 3100; 5 and 10 steps on 256^2 .. 512^2).
-  double tile_cycles(const Group& G, int K, int ty, int tx, int64_t tiles) const {
+  // and two per launch, with prologues of 3, 8 and 14 arrays, on 500 x 513 ..
+  // 3000 x 3100; 5 and 10 steps on 256^2 .. 512^2).
+  double tile_cycles(const Group& G, int K, int ty, int tx, int64_t tiles, bool pro = false) const {
     const int64_t per = (tiles + kSMs - 1) / kSMs;  // tiles of one SM
     const int pts = (int)G.offsets.size() / 3;
     const int ry = G.radius[1], rx = G.radius[2];
@@ -722,6 +738,7 @@ struct Planner {
       else t += parallel * (290.0 * pts / 5 + 0.6 * epi) * std::ceil(cells / 256);
     }
     if (f64) t += per * 350;
+    if (pro && f64) t += per * (double)(ty + 2 * K * ry) * (tx + 2 * K * rx) * pro_cycles(G) / 128 / 2;
     return t;
   }
   int64_t tiles_of(const std::vector<int64_t>& shape, int ty, int tx) const {
@@ -846,33 +863,56 @@ struct Planner {
     int64_t seg = 0;
     int nw = 4;
     if (G.kind == GroupKind::Stencil && var == 1 && cells > 0) {
-      // (the last launch of an uneven split runs fewer steps)
-      auto total = [&](double cycles, int K) { return cycles * S / K + launch * ((S + K - 1) / K); };
-      double best = total(stream_cycles(G, G.depth, seg, nw), G.depth);
+      // (the last launch of an uneven split runs fewer steps; the first alone
+      // evaluates a prologue, which binary32 counts in every launch: it then
+      // takes deeper ones, 9 steps on the sum of 8 arrays of 3000 x 3100 82 us in
+      // one launch against 94 in two)
+      auto total = [&](double cycles, double first, int K) {
+        return first - cycles + std::max(1.0, (double)S / K) * cycles + launch * ((S + K - 1) / K);
+      };
+      auto stream_total = [&](int K, int64_t& sg, int& n) {
+        int64_t sg1;
+        int n1;
+        const bool pro = !G.members.empty();
+        const double first = stream_cycles(G, K, pro, sg, n);
+        if (K == S || !pro || G.dtype != DCP_F64) return total(first, first, K);
+        const double rest = stream_cycles(G, K, false, sg1, n1);
+        sg = sg1, n = n1;
+        return total(rest, first, K);
+      };
+      double best = stream_total(G.depth, seg, nw);
       if (free_depth)
         for (int most = 1; most <= std::min(S, G.dtype == DCP_F32 ? 10 : 4); ++most) {
           const int K = even(most);
           int64_t sg;
           int n;
           if (!stream_eligible(G, K)) continue;
-          const double c = total(stream_cycles(G, K, sg, n), K);
+          const double c = stream_total(K, sg, n);
           if (c < best) best = c, G.depth = K, seg = sg, nw = n;
         }
       // Small grids run faster in shared-memory tiles, where every cell of a
       // step is in flight at once (256^2 binary64, 24 steps: 46 us against 91;
       // 64^2 binary32: 17 against 25).  From 512^2 on the stream wins, but for
-      // periodic binary64 grids: a step whose sums share no pairs pays for the
-      // strip's halo columns (1000 x 1001, 9 points of radius 2, 7 steps: 191 us
-      // streamed, 156 in tiles) and a narrow one for idle lanes.
+      // prologues of many arrays, whose rings leave few warps (the step of a sum
+      // of 8 arrays of 1000 x 1001, periodic: binary32 14 us streamed, 8 in
+      // tiles, binary64 45 and 31), and for periodic binary64 grids: a step
+      // whose sums share no pairs pays for the strip's halo columns (1000 x
+      // 1001, 9 points of radius 2, 7 steps: 191 us streamed, 156 in tiles) and
+      // a narrow one for idle lanes.
       const bool small = cells <= 512 * 512, f64 = G.dtype == DCP_F64;
       const bool periodic = G.bc == DCP_BC_PERIODIC;
-      if (nd == 2 && (small || (f64 && periodic)) && !has(DCP_OPT_STENCIL_KERNEL) &&
+      const int64_t n_in = arrays_in(G);
+      const bool many = f64 ? n_in >= 3
+                            : periodic && n_in >= 6 && cells >= 1 << 17 && S <= 4 &&
+                                  (S == 1 || cells * S <= 5000000 || (S == 2 && n_in >= 8));
+      if (nd == 2 && (small || many || (f64 && periodic)) && !has(DCP_OPT_STENCIL_KERNEL) &&
           !has(DCP_OPT_TILE_X) && !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS)) {
-        for (int most = 1; most <= std::min(S, small ? 12 : 4); ++most) {
+        const bool fixed = !small || (!f64 && many);  // the default tile
+        for (int most = 1; most <= std::min(S, fixed ? 4 : 12); ++most) {
           const int K = free_depth ? even(most) : G.depth;
-          for (int tx : small ? std::vector<int>{16, 32} : std::vector<int>{32}) {
+          for (int tx : fixed ? std::vector<int>{f64 ? 32 : 64} : std::vector<int>{16, 32}) {
             std::vector<int> heights = {16, 32};
-            if (small) {
+            if (!fixed) {
               heights = {4, 8, 12, 16, 24, 32};
               // heights that give every SM the same number of tiles, one or two
               // (256 rows in 8 strips: 14, 152 tiles; 16 rows would leave 24 SMs idle)
@@ -887,9 +927,13 @@ struct Planner {
               const long smem = 2L * (ty + 2 * K * G.radius[1]) * (tx + 2 * K * G.radius[2]) * dtype_size(G.dtype);
               if (smem > 96 * 1024) continue;
               const int64_t tiles = tiles_of(G.shape, ty, tx);
-              const double c = total(tile_cycles(G, K, ty, tx, tiles), K) + 0.3 * launch * ((S + K - 1) / K);
-              // (on large grids more than two steps only for a gain the model resolves)
-              if (c < best * (small || K <= 2 || var == 1 ? 1.0 : 0.97)) {
+              const double rest = tile_cycles(G, K, ty, tx, tiles);
+              const double first = G.members.empty() ? rest : tile_cycles(G, K, ty, tx, tiles, true);
+              const double c = total(rest, first, K) + 0.3 * launch * ((S + K - 1) / K);
+              // (on large grids more than two steps only for a gain the model
+              // resolves; binary32 takes tiles for a few steps on many inputs
+              // whatever the model says, which has no term for the inputs)
+              if (c < best * (small || K <= 2 || var == 1 ? 1.0 : 0.97) || (!f64 && many && K == S && ty == 32)) {
                 best = c;
                 var = 0;
                 G.depth = K;

@@ -40,6 +40,14 @@ def test_narrow_periodic_binary64_grids_run_in_tiles():
         assert grp["kernel_form"] == "tile"
 
 
+@pytest.mark.parametrize("shape", [(500, 513), (1000, 1001)])
+def test_steps_on_many_arrays_run_in_tiles(shape):
+    assert _stencil(shape, "f32", "periodic", 1, arrays=8)[0]["kernel_form"] == "tile"
+    assert _stencil(shape, "f64", "zero", 1, arrays=8)[0]["kernel_form"] == "tile"
+    # long runs stream: their first launch alone reads the arrays
+    assert _stencil((1000, 1001), "f32", "periodic", 9, arrays=8)[0]["kernel_form"] == "stream"
+
+
 def test_one_step_on_a_small_binary64_grid_takes_large_tiles():
     """4 x 16 cells keep a quarter of a CTA's threads busy."""
     grp, _ = _stencil((500, 513), "f64", "periodic", 1)
