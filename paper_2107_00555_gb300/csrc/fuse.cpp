@@ -640,8 +640,8 @@ struct Planner {
   // cycles per level and 42 per row with a latency of 45 per level and 130
   // per row; binary64 is bound by the FP64 pipe (p operations on 2 columns),
   // with a latency of 500 per level and 300 per row.
-  // With `pro` the launch evaluates the group's prologue.
-  double stream_cycles(const Group& G, int K, bool pro, int64_t& seg, int& nw) const {
+  // With `pro` the launch evaluates the group's prologue; ctas: CTAs of it.
+  double stream_cycles(const Group& G, int K, bool pro, int64_t& seg, int& nw, int64_t& ctas) const {
     const int64_t ny = G.shape.size() == 2 ? G.shape[0] : 1, nx = G.shape.back();
     const int ry = G.shape.size() == 2 ? G.radius[1] : 0;
     const int W = stream_width(G, K);
@@ -677,9 +677,15 @@ struct Planner {
       const int nn = (int)std::min<int64_t>(per, n);
       const double busy = G.dtype == DCP_F64 ? (nn == 1 ? 0.7 : 0.85) : 1.0;
       const double c = std::max(mem, (double)waves * (sg + 2 * K * ry) * std::max(latency, issue * nn / busy));
-      if (c < best * 0.999) best = c, seg = sg, nw = n;
+      if (c < best * 0.999) best = c, seg = sg, nw = n, ctas = items;
     }
     return best;
+  }
+
+  // Cycles the tickets of a launch's CTAs take where it reduces: about 7 ns
+  // each, those of the first few hundred beside the other CTAs' work.
+  double ticket_cycles(const Group& G, int64_t ctas) const {
+    return G.reds.empty() ? 0 : 14.0 * std::max<int64_t>(0, ctas - 512);
   }
 
   // Cycles of one batched launch of K steps with seg rows per work item: the
@@ -779,7 +785,8 @@ struct Planner {
     const double padded = (double)nz * ((ny + 7) / 8 * 8) * ((nx + 31) / 32 * 32);
     best = 0.95 * S *
            ((f64 ? std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / (2 * kSMs) + 3000)
-                 : std::max(mem, 3.84e-3 * padded * (0.6 + 0.4 * pts / 7 + epi / 252) + 5000)) + 6200);
+                 : std::max(mem, 3.84e-3 * padded * (0.6 + 0.4 * pts / 7 + epi / 252) + 5000)) + 6200) +
+           (f64 ? 0 : ticket_cycles(G, (nz + 15) / 16 * ((ny + 7) / 8) * ((nx + 31) / 32)));
     const int lx0 = G.lx, cy0 = G.cy;
     const bool odd = nx % 4 != 0;
     bool column = false;
@@ -813,7 +820,8 @@ struct Planner {
               const int64_t nn = std::min<int64_t>(per, n);
               const double c = (std::max(mem, waves * (double)(sg + ends) *
                                                   std::max(latency, issue * nn * busy * (f64 && nn == 1 ? 1.3 : 1.0))) +
-                                6200) * ((S + K - 1) / K);
+                                6200) * ((S + K - 1) / K) +
+                               (f64 ? 0 : ticket_cycles(G, items / (K * cy < 8 ? 4 : 1)));
               if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
               if (segs >= nz) break;
             }
@@ -870,15 +878,16 @@ struct Planner {
       auto total = [&](double cycles, double first, int K) {
         return first - cycles + std::max(1.0, (double)S / K) * cycles + launch * ((S + K - 1) / K);
       };
+      const int wpc = G.reds.empty() ? 1 : G.dtype == DCP_F32 ? 4 : 2;  // warps per CTA of a launch that reduces
       auto stream_total = [&](int K, int64_t& sg, int& n) {
-        int64_t sg1;
+        int64_t ctas = 0, sg1;
         int n1;
         const bool pro = !G.members.empty();
-        const double first = stream_cycles(G, K, pro, sg, n);
-        if (K == S || !pro || G.dtype != DCP_F64) return total(first, first, K);
-        const double rest = stream_cycles(G, K, false, sg1, n1);
+        const double first = stream_cycles(G, K, pro, sg, n, ctas);
+        if (K == S || !pro || G.dtype != DCP_F64) return total(first, first, K) + ticket_cycles(G, ctas / wpc);
+        const double rest = stream_cycles(G, K, false, sg1, n1, ctas);
         sg = sg1, n = n1;
-        return total(rest, first, K);
+        return total(rest, first, K) + ticket_cycles(G, ctas / wpc);
       };
       double best = stream_total(G.depth, seg, nw);
       if (free_depth)
@@ -929,7 +938,7 @@ struct Planner {
               const int64_t tiles = tiles_of(G.shape, ty, tx);
               const double rest = tile_cycles(G, K, ty, tx, tiles);
               const double first = G.members.empty() ? rest : tile_cycles(G, K, ty, tx, tiles, true);
-              const double c = total(rest, first, K) + 0.3 * launch * ((S + K - 1) / K);
+              const double c = total(rest, first, K) + 0.3 * launch * ((S + K - 1) / K) + ticket_cycles(G, tiles);
               // (on large grids more than two steps only for a gain the model
               // resolves; binary32 takes tiles for a few steps on many inputs
               // whatever the model says, which has no term for the inputs)
