@@ -715,7 +715,8 @@ struct Planner {
       longest = std::max(longest, std::min<int64_t>(ny, seg) + 2 * K * ry);
       bytes += 2.0 * ny * nx * dtype_size(G.dtype);
     }
-    const double n = std::min(4.0, items / (double)kSchedulers);
+    // (binary64: the other warps of the scheduler keep its FP64 pipe busy)
+    const double n = f64 ? 1.0 : std::min(4.0, items / (double)kSchedulers);
     const double c = std::max(rows * issue / kSchedulers + 0.5 * longest * std::max(latency, n * issue),
                               longest * latency);
     return std::max(c, bytes / (bytes > 100e6 ? 3237.0 : 6500.0));
@@ -967,6 +968,17 @@ struct Planner {
           if (c < best) best = c, G.depth = K, seg = sg;
         }
       }
+      // small periodic binary64 batches in tiles (64 instances of 32^2 to 64^2,
+      // 20 steps: 153 us streamed, 124 in tiles)
+      if (G.bc == DCP_BC_PERIODIC && G.dtype == DCP_F64 && !has(DCP_OPT_STENCIL_KERNEL) &&
+          !has(DCP_OPT_TILE_X) && !has(DCP_OPT_TILE_Y) && !has(DCP_OPT_STREAM_ROWS))
+        for (int most = most0; most <= std::min(most1, 2); ++most) {
+          const int K = free_depth ? even(most) : G.depth;
+          int64_t tiles = 0;
+          for (int m : G.batch_members) tiles += tiles_of(batch_store[m].shape, G.tile[1], G.tile[2]);
+          const double c = (tile_cycles(G, K, G.tile[1], G.tile[2], tiles) * S / K + 1.3 * launch * ((S + K - 1) / K));
+          if (c < best) best = c, var = 0, G.depth = K;
+        }
     }
     if (it != g.options.end() && it->second == 2 && G.kind == GroupKind::Stencil &&
         G.shape.size() <= 2) {

@@ -60,6 +60,12 @@ def test_tile_heights_follow_the_number_of_sms():
     assert grp["kernel_form"] == "tile" and grp["tile"][1:] == [27, 32]
 
 
+def test_small_periodic_binary64_batches_run_in_tiles():
+    sides = [32 + k % 33 for k in range(64)]
+    g = programs.batch2d(sides, 20, "periodic", "f64", fuse=C.DCP_FUSE_ALL | C.DCP_BATCH)
+    assert g.plan()["groups"][0]["kernel_form"] == "tile"
+
+
 def test_launches_that_reduce_share_tickets_between_binary32_warps():
     grp, launches = _stencil((1000, 1001), "f32", "zero", 14, reduced=True)
     assert grp["kernel_form"] == "stream" and grp["threads"] == 32
