@@ -898,7 +898,9 @@ struct Planner {
           int n;
           if (!stream_eligible(G, K)) continue;
           const double c = stream_total(K, sg, n);
-          if (c < best) best = c, G.depth = K, seg = sg, nw = n;
+          // (strips of 1-D binary64 arrays: 24 steps of 10^7 elements, fixed ring,
+          // 1.50 ms two at a time, 1.55 three, which the model holds equal)
+          if (c < best * (stream_exact(G) && K > 2 ? 0.97 : 1.0)) best = c, G.depth = K, seg = sg, nw = n;
         }
       // Small grids run faster in shared-memory tiles, where every cell of a
       // step is in flight at once (256^2 binary64, 24 steps: 46 us against 91;
