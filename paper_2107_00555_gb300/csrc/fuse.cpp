@@ -781,57 +781,57 @@ struct Planner {
     int bcy = 4, blx = 32;
     int64_t bseg = 1;
     // the shared-memory planes: whole tiles of 8 x 32 cells, one operation more
-    double best = 1e300;
     // (binary32: 63 instructions per cell, 3.84e-3 cycles of the whole GPU)
     const double padded = (double)nz * ((ny + 7) / 8 * 8) * ((nx + 31) / 32 * 32);
-    best = 0.95 * S *
-           ((f64 ? std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / (2 * kSMs) + 3000)
+    double best =
+        0.95 * S *
+            ((f64 ? std::max(mem, 1.12 * padded * (pts - 1 + epi / 128) / (2 * kSMs) + 3000)
                  : std::max(mem, 3.84e-3 * padded * (0.6 + 0.4 * pts / 7 + epi / 252) + 5000)) + 6200) +
            (f64 ? 0 : ticket_cycles(G, (nz + 15) / 16 * ((ny + 7) / 8) * ((nx + 31) / 32)));
     const int lx0 = G.lx, cy0 = G.cy;
     const bool odd = nx % 4 != 0;
     bool column = false;
     const int K = kmax;  // (binary32: two steps beat one at every size measured)
-      for (int lx : {32, 16})
-        for (int cy : {8, 4, 2}) {
-          if (!f64 && (cy == 8 || lx != 32)) continue;
-          G.lx = lx;
-          const int rows_w = 32 / lx * cy;  // rows per warp
-          if (rows_w > 2 && rows_w / 2 >= ny) continue;
-          const int64_t strips = (nx + column_width(G, K) - 1) / column_width(G, K);
-          const int64_t blocks = (ny + rows_w - 1) / rows_w;
-          const double rows = K == 1 ? cy : 2 * cy + 2;  // rows summed per plane, all levels
-          const double issue = f64 ? cy * (2 * 64 * (pts - 3 + (cy + 1.0) / cy) + epi) + 100
-                                   : rows * (52 + 4.0 * pts + epi) + 70 + (odd ? (cy + 2 * K) * 25 : 0);
-          const double latency = f64 ? 1500 : 900 + 700.0 * K;
-          const double ends = f64 ? 0.5 : 2.0 * K;  // planes an item pays for beside its own
-          // warps per scheduler: what the registers of the form allow without
-          // spills (512^3 binary64, 8 rows per lane: 1.22 ms per step at 2,
-          // 1.41 at 3; 300 x 333 x 381 binary32: 59 us at 3, 72 at 4)
-          const int nmax = f64 && cy == 8 ? 2 : 3;
-          for (int n = 1; n <= nmax; ++n)
-            for (int wv = 1; wv <= (n == nmax ? 16 : 1); ++wv) {  // whole waves of the resident warps
-              const int64_t segs = (int64_t)wv * n * kSchedulers / (strips * blocks);
-              if (segs < 1) continue;
-              const int64_t sg = (nz + std::min(segs, nz) - 1) / std::min(segs, nz);
-              const int64_t items = strips * blocks * ((nz + sg - 1) / sg);
-              const int64_t per = (items + kSchedulers - 1) / kSchedulers;
-              const int64_t waves = (per + n - 1) / n;
-              // (one warp alone keeps its scheduler's FP64 pipe busy 70 % of the time)
-              const int64_t nn = std::min<int64_t>(per, n);
-              const double c = (std::max(mem, waves * (double)(sg + ends) *
-                                                  std::max(latency, issue * nn * busy * (f64 && nn == 1 ? 1.3 : 1.0))) +
-                                6200) * ((S + K - 1) / K) +
-                               (f64 ? 0 : ticket_cycles(G, items / (K * cy < 8 ? 4 : 1)));
-              if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
-              if (segs >= nz) break;
-            }
-          if (strips * blocks > 16 * nmax * kSchedulers) {  // wide grids: long columns
-            const int64_t sg = std::min<int64_t>(nz, 64);
-            const double c = ((double)strips * blocks * nz / sg / kSchedulers * (sg + ends) * issue + 6200) * ((S + K - 1) / K);
+    for (int lx : {32, 16})
+      for (int cy : {8, 4, 2}) {
+        if (!f64 && (cy == 8 || lx != 32)) continue;
+        G.lx = lx;
+        const int rows_w = 32 / lx * cy;  // rows per warp
+        if (rows_w > 2 && rows_w / 2 >= ny) continue;
+        const int64_t strips = (nx + column_width(G, K) - 1) / column_width(G, K);
+        const int64_t blocks = (ny + rows_w - 1) / rows_w;
+        const double rows = K == 1 ? cy : 2 * cy + 2;  // rows summed per plane, all levels
+        const double issue = f64 ? cy * (2 * 64 * (pts - 3 + (cy + 1.0) / cy) + epi) + 100
+                                 : rows * (52 + 4.0 * pts + epi) + 70 + (odd ? (cy + 2 * K) * 25 : 0);
+        const double latency = f64 ? 1500 : 900 + 700.0 * K;
+        const double ends = f64 ? 0.5 : 2.0 * K;  // planes an item pays for beside its own
+        // warps per scheduler: what the registers of the form allow without
+        // spills (512^3 binary64, 8 rows per lane: 1.22 ms per step at 2,
+        // 1.41 at 3; 300 x 333 x 381 binary32: 59 us at 3, 72 at 4)
+        const int nmax = f64 && cy == 8 ? 2 : 3;
+        for (int n = 1; n <= nmax; ++n)
+          for (int wv = 1; wv <= (n == nmax ? 16 : 1); ++wv) {  // whole waves of the resident warps
+            const int64_t segs = (int64_t)wv * n * kSchedulers / (strips * blocks);
+            if (segs < 1) continue;
+            const int64_t sg = (nz + std::min(segs, nz) - 1) / std::min(segs, nz);
+            const int64_t items = strips * blocks * ((nz + sg - 1) / sg);
+            const int64_t per = (items + kSchedulers - 1) / kSchedulers;
+            const int64_t waves = (per + n - 1) / n;
+            // (one warp alone keeps its scheduler's FP64 pipe busy 70 % of the time)
+            const int64_t nn = std::min<int64_t>(per, n);
+            const double c = (std::max(mem, waves * (double)(sg + ends) *
+                                                std::max(latency, issue * nn * busy * (f64 && nn == 1 ? 1.3 : 1.0))) +
+                              6200) * ((S + K - 1) / K) +
+                             (f64 ? 0 : ticket_cycles(G, items / (K * cy < 8 ? 4 : 1)));
             if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
+            if (segs >= nz) break;
           }
+        if (strips * blocks > 16 * nmax * kSchedulers) {  // wide grids: long columns
+          const int64_t sg = std::min<int64_t>(nz, 64);
+          const double c = ((double)strips * blocks * nz / sg / kSchedulers * (sg + ends) * issue + 6200) * ((S + K - 1) / K);
+          if (c < best * 0.999) best = c, G.depth = K, bcy = cy, blx = lx, bseg = sg, column = true;
         }
+      }
     G.lx = lx0;
     G.cy = cy0;
     if (!column) return;

@@ -277,8 +277,9 @@ __device__ __forceinline__ void dcp_arrive(DcpState<N>& st, T (&out)[N][C], int 
                                            const DcpItem& it, unsigned ringc,
                                            const T (&km)[DCP_NK], Get&& get, Sides&& sides) {
   // fixed ring: a cell's sum is its own value (set on its plane's arrival,
-  // kept when the next plane finishes it)
+  // kept when the next plane finishes it); deferred runs, the pair form, have none
   constexpr bool RINGM = DCP_BC == DCP_BC_FIXED_RING;
+  static_assert(!(DCP_PAIRS && RINGM), "a deferred run has no fixed ring");
   const bool rz0 = RINGM && (j < 1 || j >= it.nz - 1), rz1 = RINGM && (j - 1 < 1 || j - 1 >= it.nz - 1);
   auto ring = [&](int r, bool rz) -> unsigned {
     return rz || y + r < 1 || y + r >= it.ny - 1 ? ~0u : ringc;
@@ -297,18 +298,13 @@ __device__ __forceinline__ void dcp_arrive(DcpState<N>& st, T (&out)[N][C], int 
     if (r > 0) {
       dcp_finish<S, 0>(out[r - 1], st.acc[r - 1], d, km);
 #pragma unroll
-      for (int c = 0; c < C; ++c) {
-        if (RINGM && ((ring(r - 1, rz1) >> c) & 1u)) out[r - 1][c] = st.acc[r - 1][c];
+      for (int c = 0; c < C; ++c)
         if (!LAST) st.acc[r - 1][c] = pend[c];
-      }
     }
     if (r < N && !LAST) {
       T l, rt;
       sides(r, cur, l, rt);
       dcp_inner<S, 0>(pend, d, cur.v, l, rt, km);
-#pragma unroll
-      for (int c = 0; c < C; ++c)
-        if (RINGM && ((ring(r, rz0) >> c) & 1u)) pend[c] = cur.v[c];
     }
 #pragma unroll
     for (int c = 0; c < C; ++c) st.before[r][c] = cur.v[c];
