@@ -185,7 +185,7 @@ class Graph:
         keep = (list(inputs), list(outputs))
 
         def run(stream=None):
-            C._check("dcp_run", lib.dcp_run(h, ins, outs, _raw_stream(stream)))
+            C._check("dcp_run", lib.dcp_run(h, ins, outs, _raw_stream(stream or None)))
             return keep[1]
 
         run.outputs = outputs
