@@ -455,7 +455,7 @@ static void launch_axis(GraphImpl& g, LaunchSpec& ls, const std::vector<const vo
   const int64_t base = (outer + TO - 1) / TO * ntiles;
   // (a split takes at least 32 loads per thread; a few rows of no whole number
   // of vectors 32 elements: the sum of 16 binary32 arrays of 3 x 1000003 along
-  // its rows 111 -> 77 us)
+  // its rows 111 -> 41 us)
   const int64_t least = TR * 32 * (R % rv == 0 || base >= rt.sms ? rv : 1);
   int64_t S = 1;
   if (base < target && R > least)
