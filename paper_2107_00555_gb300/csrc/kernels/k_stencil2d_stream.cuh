@@ -19,10 +19,11 @@
 //
 // Measured on a GB300 against the form that kept 2*RY + 1 rows per level and
 // read them element by element (with the planner's depth and rows per item):
-// 4000 x 4100 binary32, fixed ring, 50 steps 526 -> 295 us; 2047 x 2051
-// binary64, periodic, 20 steps 721 (shared-memory tiles) -> 572 us; 4096
-// binary32 instances of 32^2 to 512^2, 20 steps 2.84 -> 2.01 ms; the 20-step
-// reverse pass of a 4096^2 binary32 chain with its loss 3.01 -> 1.71 ms.
+// 4000 x 4100 binary32, fixed ring, 50 steps 526 -> 291 us; 2047 x 2051
+// binary64, periodic, 20 steps 723 (shared-memory tiles) -> 567 us; 4096
+// binary32 instances of 32^2 to 512^2, 20 steps 2.84 -> 1.83 ms; the 20-step
+// reverse pass of a 4096^2 binary32 chain with its loss 3.01 -> 1.69 ms; four
+// steps of 10^8 binary32 elements, zero boundary, 242 -> 209 us.
 //
 // Work items are (array, strip, row segment); a segment streams its rows plus
 // NSTEPS*RY warm-up rows above and below it.  Warps stride through the items
@@ -44,8 +45,10 @@
 // shuffles for 128 columns.
 //
 // The generated prefix defines DCP_T, DCP_C, DCP_RX, DCP_RY, DCP_NSTEPS,
-// DCP_BC, DCP_THREADS, DCP_KNAME, DCP_BATCH, DCP_LAST, DCP_R, DCP_GUARD, DCP_MINB,
-// DCP_W, DCP_HX, DCP_VEC (elements per access, 0: per instance), DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions after the last step), DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
+// DCP_BC, DCP_THREADS, DCP_KNAME, DCP_BATCH, DCP_LAST, DCP_R, DCP_GUARD,
+// DCP_MINB, DCP_W, DCP_HX, DCP_VEC (elements per access, 0: per instance),
+// DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions
+// after the last step), DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
 //   T    dcp_pro(const T (&ld)[DCP_NIN], const T* sc)     input maps on the loaded values
 //   struct DcpRow<L>::run<RINGM>(a, st, out, km, rm)      arrival of row a in level L+1
 //   T    dcp_epi<L>(T v)                 epilogue maps fused after step L
