@@ -142,15 +142,15 @@ Ex ex_op(int op, int dtype, double imm_v, const Ex& a, const Ex& b) {
     r.x = x;
     r.y = y;
   };
-  // p + q or p - q.  Only a product read here alone is fused: one that others
-  // read too has its rounded value, and the difference of a product with
-  // itself (or with another node of the same factors) is 0.
+  // p + q or p - q.  A product is fused into the sum, except with itself or with
+  // another node of the same factors: that difference is 0, not the rounding
+  // error of the product.
   auto sum = [&](const Ex& p, const Ex& q, bool minus) {
     auto neg = [](const std::string& v, bool n) { return n ? "dcp_neg(" + v + ")" : v; };
     const bool same = p.s == q.s || (p.mul() && q.mul() && ((p.x == q.x && p.y == q.y) || (p.x == q.y && p.y == q.x)));
-    if (!same && p.mul() && p.uses == 1)
+    if (!same && p.mul() && !(q.mul() && q.uses < p.uses))
       r.s = "dcp_fma_rn(" + neg(p.x, p.neg) + ", " + p.y + ", " + neg(q.s, minus) + ")";
-    else if (!same && q.mul() && q.uses == 1)
+    else if (!same && q.mul())
       r.s = "dcp_fma_rn(" + neg(q.x, q.neg != minus) + ", " + q.y + ", " + p.s + ")";
     else
       r.s = std::string(minus ? "dcp_sub_rn(" : "dcp_add_rn(") + p.s + ", " + q.s + ")";
