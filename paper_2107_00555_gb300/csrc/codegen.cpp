@@ -1033,7 +1033,8 @@ static CodegenOut gen_stream_kernel(const GraphImpl& g, const Group& G, int s0, 
   os << "#define DCP_RX " << rx << "\n#define DCP_RY " << ry << "\n#define DCP_NSTEPS " << nsteps
      << "\n#define DCP_R " << ring << "\n#define DCP_W " << stream_width(G, nsteps)
      << "\n#define DCP_HX " << (exact ? nsteps * rx : (nsteps * rx + C - 1) / C * C)
-     << "\n#define DCP_VEC " << vec << "\n";
+     << "\n#define DCP_VEC " << vec
+     << "\n#define DCP_HUGE " << (!batch && G.shape.back() > 0x7fffffff - 4096 ? 1 : 0) << "\n";
   const Defer guard = first ? plan_defer(g, G, 0) : Defer();
   os << "#define DCP_GUARD " << (guard.on ? 1 : 0) << "\n";
   if (G.min_ctas > 0) os << "#define DCP_MINB " << std::max(1, G.min_ctas * G.threads / threads) << "\n";

@@ -47,7 +47,7 @@
 // The generated prefix defines DCP_T, DCP_C, DCP_RX, DCP_RY, DCP_NSTEPS,
 // DCP_BC, DCP_THREADS, DCP_KNAME, DCP_BATCH, DCP_LAST, DCP_R, DCP_GUARD,
 // DCP_MINB, DCP_W, DCP_HX, DCP_VEC (elements per access, 0: per instance),
-// DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions
+// DCP_HUGE, DCP_NLOAD, DCP_NIN = max(1, DCP_NLOAD), DCP_PRO, DCP_POST (maps or reductions
 // after the last step), DCP_NSTORE, DCP_NRED, DCP_NSCALAR, dcp_red_op(r) and
 //   T    dcp_pro(const T (&ld)[DCP_NIN], const T* sc)     input maps on the loaded values
 //   struct DcpRow<L>::run<RINGM>(a, st, out, km, rm)      arrival of row a in level L+1
@@ -82,8 +82,17 @@ static_assert(R >= 4, "the ring holds a pair of rows, the pair before and one ah
 
 typedef DcpStParamsT<T> DcpStParams;
 
+// Sums of columns.  In rows within a strip of 2^31 columns (DCP_HUGE) those past
+// 2^31 - 1, beyond the row's end, come as negative numbers below any halo's.
+#if DCP_HUGE
+#define DCP_PLUS(a, b) ((int)((unsigned)(a) + (unsigned)(b)))
+#else
+#define DCP_PLUS(a, b) (a + b)
+#endif
+
 __device__ __forceinline__ int dcp_wrap(int q, int n) {
   if ((unsigned)q < (unsigned)n) return q;
+  if (DCP_HUGE && q < -(1 << 30)) return (int)((unsigned)q % (unsigned)n);
   int r = q % n;
   return r < 0 ? r + n : r;
 }
@@ -301,17 +310,17 @@ __device__ __forceinline__ void dcp_stream_impl(const DcpItem& it, Pro& pro, Out
   extern __shared__ __align__(16) unsigned char dcp_smem[];
   const int lane = threadIdx.x & 31;
   DcpCols cols;
-  const int col0 = it.x0 - HX + lane * C;
+  const int col0 = DCP_PLUS(it.x0 - HX, lane * C);
   cols.dst = (unsigned)__cvta_generic_to_shared(dcp_smem) +
              (threadIdx.x >> 5) * (DCP_NIN * R * ROWB) + lane * 16;
   cols.ring = cols.in = 0u;
   const int vec = dcp_vec<CHECK>(it);
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    const int col = col0 + c;
+    const int col = DCP_PLUS(col0, c);
     if (CHECK) cols.ring |= col < DCP_RX || col >= it.nx - DCP_RX ? 1u << c : 0u;
     cols.keep[c] = (unsigned)col < (unsigned)it.nx ? ~(typename DcpBits<T>::type)0 : 0;
-    const int u = it.x0 - HX + (lane + 32 * c) * vec;  // first column of access c
+    const int u = DCP_PLUS(it.x0 - HX, (lane + 32 * c) * vec);  // first column of access c
     cols.in |= (unsigned)u < (unsigned)it.nx ? 1u << c : 0u;
     if (CHECK && DCP_BC == DCP_BC_PERIODIC) cols.pcol[c] = dcp_wrap(u, it.nx);
   }
@@ -390,19 +399,25 @@ __device__ __forceinline__ void dcp_stream(const DcpItem& it, Pro&& pro, DcpGuar
                                            const T (&km)[DCP_NK], Output&& output) {
   const int lo = DCP_BC == DCP_BC_FIXED_RING ? DCP_RX : 0;
   const int first = it.x0 - HX;
-  if (first >= lo && first + SPAN <= it.nx - lo) dcp_stream_impl<false>(it, pro, output, guard, km);
+  if (first >= lo && (DCP_HUGE ? first <= it.nx - lo - SPAN : first + SPAN <= it.nx - lo)) dcp_stream_impl<false>(it, pro, output, guard, km);
   else dcp_stream_impl<true>(it, pro, output, guard, km);
 }
 
 // Bit c: the lane's column c is written by the strip starting at x0.
 __device__ __forceinline__ unsigned dcp_written(int x0, int nx) {
-  const int col0 = x0 - HX + (threadIdx.x & 31) * C;
   unsigned m = 0u;
+#if DCP_HUGE
+  const int at = (int)(threadIdx.x & 31) * C - HX;  // the lane's first column, from x0
+#pragma unroll
+  for (int c = 0; c < C; ++c) m |= at + c >= 0 && at + c < W && at + c < nx - x0 ? 1u << c : 0u;
+#else
+  const int col0 = x0 - HX + (threadIdx.x & 31) * C;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int col = col0 + c;
     m |= col >= x0 && col < x0 + W && col < nx ? 1u << c : 0u;
   }
+#endif
   return m;
 }
 
@@ -428,7 +443,7 @@ extern "C" __global__ void __launch_bounds__(DCP_THREADS, DCP_MINB) DCP_KNAME(co
 #pragma unroll
   for (int r = 0; r < DCP_NRED; ++r) acc[r] = dcp_red_init<T>(dcp_red_op(r));
   const int ny = p.ny, nx = p.nx;
-  const int strips = (nx + W - 1) / W;
+  const int strips = DCP_HUGE ? (nx - 1) / W + 1 : (nx + W - 1) / W;
   const int SEG = p.seg > 0 ? p.seg : ny;
   const int segs = (ny + SEG - 1) / SEG;
   const int items = strips * segs;

@@ -606,7 +606,7 @@ static void launch_stencil(GraphImpl& g, LaunchSpec& ls, const std::vector<const
       occ = ls.occ_scalar;
     }
     const int W = G.variant == 1 ? stream_width(G, ls.s1 - ls.s0) : column_width(G, ls.s1 - ls.s0);
-    int64_t items = (int64_t)((p.nx + W - 1) / W);
+    int64_t items = ((int64_t)p.nx + W - 1) / W;
     if (G.variant == 1) items *= (p.ny + G.seg - 1) / G.seg;
     else items *= (int64_t)((p.ny + 32 / G.lx * G.cy - 1) / (32 / G.lx * G.cy)) * ((p.nz + G.seg - 1) / G.seg);
     const int wpb = ls.code.threads / 32;
@@ -729,9 +729,9 @@ static void launch_batch(GraphImpl& g, LaunchSpec& ls, const std::vector<const v
       I.in = first ? ptr[M.st_in] : (const char*)in_slab + off;
       I.out = last ? const_cast<void*>(ptr[M.st_out]) : (char*)out_slab + off;
       I.ny = (int32_t)M.shape[0];
-      I.nx = (int32_t)M.shape[1];
-      I.tiles_x = (int32_t)(G.variant == 1 ? (I.nx + W - 1) / W
-                                           : (I.nx + G.tile[2] - 1) / G.tile[2]);
+      const int64_t nx = M.shape[1];
+      I.nx = (int32_t)nx;
+      I.tiles_x = (int32_t)(G.variant == 1 ? (nx + W - 1) / W : (nx + G.tile[2] - 1) / G.tile[2]);
       I.tile0 = (int32_t)t0;
       t0 += tiles_of(k);
     }
