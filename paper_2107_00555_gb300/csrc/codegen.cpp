@@ -1252,6 +1252,8 @@ bool column_eligible(const GraphImpl& g, const Group& G) {
   if (G.kind != GroupKind::Stencil || G.shape.size() != 3 || !G.members.empty()) return false;
   if (G.radius[0] != 1 || G.radius[1] > 1 || G.radius[2] > 1) return false;
   if (G.shape[1] * G.shape[2] > 0x7fffffff) return false;  // offsets within a plane are 32-bit
+  for (int64_t n : G.shape)
+    if (n > 0x7fffffff - 4096) return false;  // a block may reach past the last cell
   for (int s = 0; s < (int)G.steps.size(); ++s)
     if (!column_step(g, G, s)) return false;
   return true;

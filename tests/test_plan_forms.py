@@ -80,3 +80,12 @@ def test_deferred_weight_is_one_of_the_first_row():
     _, launches = _stencil((1000, 1001), "f64", "zero", 3, STAR2, W2)
     scales = [s for l in launches for s in l["deferred_scales"]]
     assert scales[:2] == [1, 1] and scales[2] == pytest.approx(0.05 ** 3, rel=1e-15)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_columns_leave_extents_within_a_block_of_2p31_alone(axis):
+    """A block of the last rows or columns would reach past what an int holds."""
+    shape = [1, 1, 1]
+    shape[axis] = (1 << 31) - 1
+    grp, _ = _stencil(tuple(shape), "f32", "zero", 2, programs.SEVEN_POINT, programs.SEVEN_WEIGHTS)
+    assert grp["kernel_form"] == "tile"
